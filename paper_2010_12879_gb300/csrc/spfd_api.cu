@@ -305,8 +305,9 @@ T *vcycle(spfd_ctx *c, int l, T *bl, bool proj, int nk, bool rz, bool head) {
     proj = false;
   }
   if (l == nl - 1) {
+    // slots of x that are not unknowns of the level are zero from its
+    // allocation on: nothing but this kernel writes the coarsest x
     const double m = c->m;
-    cudaMemsetAsync(lv.X<T>(), 0, lv.S * nk * sizeof(T), st);
     SPFD_LAUNCH(c, "coarsest_solve", f32, 1, (8 * m * m + 2 * w * m) * nk, 2 * m * m * nk,
                 launch_coarse_solve<T>(c->m, lv.S, c->cidx, c->Binv, bl, lv.X<T>(), st, nk));
     return lv.X<T>();
@@ -363,7 +364,7 @@ T *vcycle(spfd_ctx *c, int l, T *bl, bool proj, int nk, bool rz, bool head) {
     return cur;
   }
   T *cur = lv.X<T>(), *oth = lv.Tt<T>();
-  if (head)  // vcycle_head ran the projected first sweep already
+  if (head)  // vcycle_head or the restriction ran the first sweep already
     ;
   else if (proj)
     SPFD_LAUNCH(c, "jacobi_first_l0", f32, 1, 4 * w * S, 2 * S,
@@ -398,11 +399,16 @@ T *vcycle(spfd_ctx *c, int l, T *bl, bool proj, int nk, bool rz, bool head) {
                                      block_order(c, TF_RESID, l)));
   Level &cl = c->L[l + 1];
   const double Sc = (double)cl.S * nk;
+  // the coarse level's first sweep from the zero guess needs nothing but the
+  // value just restricted: a single right-hand side takes it along (batches
+  // keep the separate kernel, whose block order the autotuner picks)
+  const bool first = nk == 1 && !c->ord && l + 2 < nl;
   SPFD_LAUNCH(c, lvl_name(LVL_NAMES("restrict"), l), f32, 1,
-              28 * w * Sc + w * S, 54 * Sc,
+              (first ? 30 : 28) * w * Sc + w * S, 54 * Sc,
               launch_restrict<T>(lv.g, cl.g, cl.PP<T>(), lv.R<T>(), cl.B<T>(), st, nk,
-                                 block_order(c, TF_RESTRICT, l)));
-  T *ec = vcycle<T>(c, l + 1, cl.B<T>(), false, nk);
+                                 block_order(c, TF_RESTRICT, l), cl.WDINV<T>(),
+                                 first ? cl.X<T>() : nullptr));
+  T *ec = vcycle<T>(c, l + 1, cl.B<T>(), false, nk, false, first);
   SPFD_LAUNCH(c, lvl_name(LVL_NAMES("prolong"), l), f32, 1,
               (27.0 / 8.0 + 2.0) * w * S + w * Sc, 7 * S,
               launch_prolong<T>(lv.g, cl.g, lv.PC<T>(), ec, cur, st, nk,

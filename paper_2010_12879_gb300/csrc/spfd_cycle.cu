@@ -14,6 +14,8 @@
 
 namespace spfd {
 
+constexpr int CS_THREADS = 128;  // threads per block of the coarsest solve
+
 // ------------------------------------------------------------ smoothers
 // Level 0 (7-point): r = b - A x, and the weighted-Jacobi sweep
 // x_out = x + omega D^-1 (b - A x), on the row mapping.  (The level-0 row
@@ -80,14 +82,7 @@ k_jacobi7(Grid g, const C *__restrict__ gx, const T *__restrict__ diag,
   }
 }
 
-// This thread's slot in a 27-point kernel over the staged brick: with
-// compaction (FP64) the brick's n-th active slot for thread n, else the
-// thread's own slot.  mine: the thread computes the stencil at ts; idle: its
-// own slot is inactive and gets the zero-row result.
-struct SlotMap {
-  int ts;
-  bool mine, idle;
-};
+// This thread's slot in a 27-point kernel over the staged brick.
 template <typename T>
 __device__ __forceinline__ SlotMap slot_map(const ActList &al) {
   const int t = threadIdx.x;
@@ -108,7 +103,7 @@ __device__ __forceinline__ SlotMap slot_map(const ActList &al) {
 // neighbour table and activity list.  A zero row (clear activity bit) gets
 // r = b - 0 = b without its 27 coefficients or any arithmetic.  FP64:
 // thread n computes the brick's n-th active slot (compaction).
-template <typename T, bool COH>
+template <typename T>
 __device__ __forceinline__ void residual27_unit(const Grid &g, const T *__restrict__ st,
                                                 const T *x, const T *b, T *r, int bk,
                                                 T (*tl)[10][10], int *sn, ActList &al) {
@@ -118,21 +113,21 @@ __device__ __forceinline__ void residual27_unit(const Grid &g, const T *__restri
   if constexpr (compact27<T>()) {
     act_stage(g, bk, al);
     __syncthreads();
-    tile_full<T, COH>(tl, x, bk, sn);
-    if (!act_on(al, t)) r[base + t] = ldv<COH>(b + base + t);
+    tile_full<T>(tl, x, bk, sn);
+    if (!act_on(al, t)) r[base + t] = b[base + t];
     __syncthreads();
     if (t < al.pre[16]) {
       const int ts = act_slot(al, t);
       const size_t s = base + ts;
-      r[s] = ldv<COH>(b + s) - apply27_tile<T>(tl, st, S, s, ts);
+      r[s] = b[s] - apply27_tile<T>(tl, st, S, s, ts);
     }
   } else {
     const bool on = (act_word(g, bk) >> (t & 31)) & 1u;
     __syncthreads();
-    tile_full<T, COH>(tl, x, bk, sn);
+    tile_full<T>(tl, x, bk, sn);
     __syncthreads();
     const size_t s = base + t;
-    r[s] = ldv<COH>(b + s) - (on ? apply27_tile<T>(tl, st, S, s, t) : T(0));
+    r[s] = b[s] - (on ? apply27_tile<T>(tl, st, S, s, t) : T(0));
   }
 }
 
@@ -150,7 +145,7 @@ k_residual27(Grid g, const T *__restrict__ st, const T *__restrict__ x,
   const size_t S = (size_t)g.nb * BV, base = (size_t)bk * BV;
   if constexpr (rhs_tile<ORD>() == 1) {
     const size_t off = (size_t)rhs * S;
-    residual27_unit<T, false>(g, st, x + off, b + off, r + off, bk, tl[0], sn, al);
+    residual27_unit<T>(g, st, x + off, b + off, r + off, bk, tl[0], sn, al);
   } else {
     load_nbr(g, bk, sn);
     act_stage(g, bk, al);
@@ -174,7 +169,7 @@ k_residual27(Grid g, const T *__restrict__ st, const T *__restrict__ x,
 
 // One weighted-Jacobi sweep xout = xin + omega D^-1 (b - A xin) on brick bk
 // of a 27-point level (as residual27_unit; a zero row gets xin + w b).
-template <typename T, bool COH>
+template <typename T>
 __device__ __forceinline__ void jacobi27_unit(const Grid &g, const T *__restrict__ st,
                                               const T *__restrict__ wdinv, const T *xin,
                                               const T *b, T *xout, int bk, T (*tl)[10][10],
@@ -185,23 +180,23 @@ __device__ __forceinline__ void jacobi27_unit(const Grid &g, const T *__restrict
   if constexpr (compact27<T>()) {
     act_stage(g, bk, al);
     __syncthreads();
-    tile_full<T, COH>(tl, xin, bk, sn);
+    tile_full<T>(tl, xin, bk, sn);
     __syncthreads();
     if (!act_on(al, t))
-      xout[base + t] = tile_at(tl, t) + wdinv[base + t] * ldv<COH>(b + base + t);
+      xout[base + t] = tile_at(tl, t) + wdinv[base + t] * b[base + t];
     if (t < al.pre[16]) {
       const int ts = act_slot(al, t);
       const size_t s = base + ts;
-      const T r = ldv<COH>(b + s) - apply27_tile<T>(tl, st, S, s, ts);
+      const T r = b[s] - apply27_tile<T>(tl, st, S, s, ts);
       xout[s] = tile_at(tl, ts) + wdinv[s] * r;
     }
   } else {
     const bool on = (act_word(g, bk) >> (t & 31)) & 1u;
     __syncthreads();
-    tile_full<T, COH>(tl, xin, bk, sn);
+    tile_full<T>(tl, xin, bk, sn);
     __syncthreads();
     const size_t s = base + t;
-    const T r = ldv<COH>(b + s) - (on ? apply27_tile<T>(tl, st, S, s, t) : T(0));
+    const T r = b[s] - (on ? apply27_tile<T>(tl, st, S, s, t) : T(0));
     xout[s] = tile_at(tl, t) + wdinv[s] * r;
   }
 }
@@ -221,7 +216,7 @@ k_jacobi27(Grid g, const T *__restrict__ st, const T *__restrict__ wdinv,
   const size_t S = (size_t)g.nb * BV, base = (size_t)bk * BV;
   if constexpr (rhs_tile<ORD>() == 1) {
     const size_t off = (size_t)rhs * S;
-    jacobi27_unit<T, false>(g, st, wdinv, xin + off, b + off, xout + off, bk, tl[0], sn, al);
+    jacobi27_unit<T>(g, st, wdinv, xin + off, b + off, xout + off, bk, tl[0], sn, al);
   } else {
     load_nbr(g, bk, sn);
     act_stage(g, bk, al);
@@ -403,7 +398,7 @@ k_cheb(size_t S, const T *__restrict__ wdinv, const T *__restrict__ r, T *__rest
 // the 8 child bricks (16^3 nodes, fs[1..16]^3) as 16-byte vectors, then the
 // three planes fs[0][*][*], fs[1..16][0][*] and fs[1..16][1..16][0] from the
 // bricks before them, one value per thread.
-template <typename T, bool COH>
+template <typename T>
 __device__ __forceinline__ void restrict_fill(T (*fs)[17][17], const T *src, const int *sk) {
   constexpr int VN = 16 / (int)sizeof(T);  // values per vector
   constexpr int VPB = BV / VN;             // vectors per brick
@@ -415,8 +410,7 @@ __device__ __forceinline__ void restrict_fill(T (*fs)[17][17], const T *src, con
     V16<T> v;
     if (nb >= 0) {
       const T *p = src + (size_t)nb * BV + e0;
-      if constexpr (COH) *reinterpret_cast<uint4 *>(&v) = __ldcg(reinterpret_cast<const uint4 *>(p));
-      else v = ld16(p);
+      v = ld16(p);
     } else {
 #pragma unroll
       for (int i = 0; i < VN; ++i) v.v[i] = T(0);
@@ -438,8 +432,7 @@ __device__ __forceinline__ void restrict_fill(T (*fs)[17][17], const T *src, con
     }
     const int nb = sk[((fz + 7) >> 3) * 9 + ((fy + 7) >> 3) * 3 + ((fx + 7) >> 3)];
     fs[fz][fy][fx] = nb >= 0
-        ? ldv<COH>(&src[(size_t)nb * BV + (((fz - 1) & 7) * 8 + ((fy - 1) & 7)) * 8 +
-                        ((fx - 1) & 7)])
+        ? src[(size_t)nb * BV + (((fz - 1) & 7) * 8 + ((fy - 1) & 7)) * 8 + ((fx - 1) & 7)]
         : T(0);
   }
 }
@@ -447,17 +440,18 @@ __device__ __forceinline__ void restrict_fill(T (*fs)[17][17], const T *src, con
 // One coarse brick bk, one coarse node per thread (NT threads call it).  A
 // coarse node whose interpolation column is zero (clear activity bit)
 // restricts to exactly +0: its 27 weights are not read.
-template <typename T, bool COH>
+template <typename T>
 __device__ __forceinline__ void restrict_unit(const Grid &gc, size_t Sf, const T *__restrict__ P,
                                               const T *rf, T *bcoarse, int bk,
-                                              T (*fs)[17][17], int *sk) {
+                                              T (*fs)[17][17], int *sk,
+                                              const T *__restrict__ wdinv, T *xc) {
   const int t = threadIdx.x;
   const size_t Sc = (size_t)gc.nb * BV, s = (size_t)bk * BV + t;
   const int cx = 2 * (t & 7) + 1, cy = 2 * ((t >> 3) & 7) + 1, cz = 2 * (t >> 6) + 1;
   if (t < 27) sk[t] = gc.kid[(size_t)bk * 27 + t];
   const bool on = (act_word(gc, bk) >> (t & 31)) & 1u;
   __syncthreads();
-  restrict_fill<T, COH>(fs, rf, sk);
+  restrict_fill<T>(fs, rf, sk);
   __syncthreads();
   T acc = 0;
   if (on) {
@@ -468,12 +462,13 @@ __device__ __forceinline__ void restrict_unit(const Grid &gc, size_t Sf, const T
     }
   }
   bcoarse[s] = acc;
+  if (xc) xc[s] = wdinv[s] * acc;
 }
 
 template <typename T, int ORD>
 __global__ void __launch_bounds__(NT)
 k_restrict(Grid gc, size_t Sf, const T *__restrict__ P, const T *__restrict__ rf,
-           T *__restrict__ bcoarse, int nk) {
+           T *__restrict__ bcoarse, int nk, const T *__restrict__ wdinv, T *__restrict__ xc) {
   pdl_entry();
   __shared__ T fs[17][17][17];
   __shared__ int sk[27];
@@ -482,8 +477,8 @@ k_restrict(Grid gc, size_t Sf, const T *__restrict__ P, const T *__restrict__ rf
   const int t = threadIdx.x;
   const size_t Sc = (size_t)gc.nb * BV, s = (size_t)bk * BV + t;
   if constexpr (rhs_tile<ORD>() == 1) {
-    restrict_unit<T, false>(gc, Sf, P, rf + (size_t)rhs * Sf, bcoarse + (size_t)rhs * Sc, bk,
-                            fs, sk);
+    restrict_unit<T>(gc, Sf, P, rf + (size_t)rhs * Sf, bcoarse + (size_t)rhs * Sc, bk,
+                            fs, sk, wdinv, xc);
   } else {
     const int cx = 2 * (t & 7) + 1, cy = 2 * ((t >> 3) & 7) + 1, cz = 2 * (t >> 6) + 1;
     if (t < 27) sk[t] = gc.kid[(size_t)bk * 27 + t];
@@ -496,7 +491,7 @@ k_restrict(Grid gc, size_t Sf, const T *__restrict__ P, const T *__restrict__ rf
     const int nr = min(rhs_tile<ORD>(), nk - rhs);
     for (int k = 0; k < nr; ++k) {
       __syncthreads();  // sk is loaded / the previous tile is consumed
-      restrict_fill<T, false>(fs, rf + (size_t)(rhs + k) * Sf, sk);
+      restrict_fill<T>(fs, rf + (size_t)(rhs + k) * Sf, sk);
       __syncthreads();
       T acc = 0;
 #pragma unroll
@@ -517,24 +512,21 @@ k_restrict(Grid gc, size_t Sf, const T *__restrict__ P, const T *__restrict__ rf
 // 8 fine values as 2-vectors along x, then writes the 8 corrected values.
 // No shared memory and no barrier: every load is independent.
 // Pair `pair` of fine bricks, thread `tid` (0..127) of the pair's group;
-// nr right-hand sides from rhs on (S apart on each level).
-template <typename T, bool COH>
+// nr right-hand sides from rhs on (S apart on each level).  The weights and
+// the corners' slots are in registers before the wait.
+template <typename T>
 __device__ __forceinline__ void prolong_unit(const Grid &gf, const Grid &gc,
                                              const T *__restrict__ Pc, const T *ec, T *ef,
                                              int pair, int tid, int rhs, int nr) {
-  const int bk = pair * 2 + (tid >> 6);
-  if (bk >= gf.nb) return;
-  const int cell = tid & 63;
+  const int bk = pair * 2 + (tid >> 6), cell = tid & 63;
   const int ccx = cell & 3, ccy = (cell >> 2) & 3, ccz = cell >> 4;
   const size_t NC = (size_t)gf.nb * 64, cid = (size_t)bk * 64 + cell;
   T w[27];
+  int es[8];
+  if (bk < gf.nb) {
 #pragma unroll
-  for (int j = 0; j < 27; ++j) w[j] = Pc[(size_t)j * NC + cid];
-  const int4 bc = gf.bco[bk];
-  for (int k = 0; k < nr; ++k) {
-    const T *ecj = ec + (size_t)(rhs + k) * gc.nb * BV;
-    T *efj = ef + (size_t)(rhs + k) * gf.nb * BV;
-    T e[8];
+    for (int j = 0; j < 27; ++j) w[j] = Pc[(size_t)j * NC + cid];
+    const int4 bc = gf.bco[bk];
 #pragma unroll
     for (int o = 0; o < 8; ++o) {
       const int gx_ = 4 * bc.x + ccx + (o & 1), gy_ = 4 * bc.y + ccy + ((o >> 1) & 1),
@@ -542,67 +534,116 @@ __device__ __forceinline__ void prolong_unit(const Grid &gf, const Grid &gc,
       const int pb = (((gz_ >> 3) - (bc.z >> 1)) << 2) | (((gy_ >> 3) - (bc.y >> 1)) << 1) |
                      ((gx_ >> 3) - (bc.x >> 1));
       const int nb = __ldg(&gf.par[(size_t)bk * 8 + pb]);
-      e[o] = nb >= 0 ? ldv<COH>(&ecj[(size_t)nb * BV + ((gz_ & 7) * 8 + (gy_ & 7)) * 8 +
-                                     (gx_ & 7)])
-                     : T(0);
+      es[o] = nb >= 0 ? nb * BV + ((gz_ & 7) * 8 + (gy_ & 7)) * 8 + (gx_ & 7) : -1;
     }
+  }
+  pdl_wait();
+  if (bk >= gf.nb) return;
+  for (int k = 0; k < nr; ++k) {
+    const T *ecj = ec + (size_t)(rhs + k) * gc.nb * BV;
+    T *efj = ef + (size_t)(rhs + k) * gf.nb * BV;
+    T e[8], v[4][2];
+    // every load is issued before the first store (ec and ef could alias as
+    // far as the compiler knows)
 #pragma unroll
     for (int r = 0; r < 4; ++r) {  // r = uz*2 + uy: one 2-vector (ux = 0, 1) per row
+      const T *row = efj + (size_t)bk * BV + ((2 * ccz + (r >> 1)) * 8 + 2 * ccy + (r & 1)) * 8 +
+                     2 * ccx;
+      if constexpr (sizeof(T) == 4) {
+        const float2 u = *reinterpret_cast<const float2 *>(row);
+        v[r][0] = u.x; v[r][1] = u.y;
+      } else {
+        const double2 u = *reinterpret_cast<const double2 *>(row);
+        v[r][0] = u.x; v[r][1] = u.y;
+      }
+    }
+#pragma unroll
+    for (int o = 0; o < 8; ++o) e[o] = es[o] >= 0 ? ecj[es[o]] : T(0);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
       const int uy = r & 1, uz = r >> 1;
       T *row = efj + (size_t)bk * BV + ((2 * ccz + uz) * 8 + 2 * ccy + uy) * 8 + 2 * ccx;
-      T v[2];
-      if constexpr (sizeof(T) == 4) {
-        const float2 u = ldv<COH>(reinterpret_cast<const float2 *>(row));
-        v[0] = u.x; v[1] = u.y;
-      } else {
-        const double2 u = ldv<COH>(reinterpret_cast<const double2 *>(row));
-        v[0] = u.x; v[1] = u.y;
-      }
 #pragma unroll
       for (int ux = 0; ux < 2; ++ux) {
         const int q = uz * 4 + uy * 2 + ux;
 #pragma unroll
         for (int o = 0; o < 8; ++o)
-          if ((o & ~q) == 0) v[ux] += w[pc_off(q) + crank(q, o)] * e[o];
+          if ((o & ~q) == 0) v[r][ux] += w[pc_off(q) + crank(q, o)] * e[o];
       }
-      if constexpr (sizeof(T) == 4) *reinterpret_cast<float2 *>(row) = make_float2(v[0], v[1]);
-      else *reinterpret_cast<double2 *>(row) = make_double2(v[0], v[1]);
+      if constexpr (sizeof(T) == 4)
+        *reinterpret_cast<float2 *>(row) = make_float2(v[r][0], v[r][1]);
+      else *reinterpret_cast<double2 *>(row) = make_double2(v[r][0], v[r][1]);
     }
   }
 }
 
 template <typename T, int ORD>
 __global__ void __launch_bounds__(128)
-k_prolong(Grid gf, Grid gc, const T *__restrict__ Pc, const T *__restrict__ ec,
-          T *__restrict__ ef, int nk) {
-  pdl_entry();
+k_prolong(Grid gf, Grid gc, const T *__restrict__ Pc, const T *ec, T *ef, int nk) {
+  pdl_trigger();
   int pair, rhs;
   unit_rhs<ORD>(nk, pair, rhs);
   const int nr = rhs_tile<ORD>() == 1 ? 1 : min(rhs_tile<ORD>(), nk - rhs);
-  prolong_unit<T, false>(gf, gc, Pc, ec, ef, pair, threadIdx.x, rhs, nr);
+  prolong_unit<T>(gf, gc, Pc, ec, ef, pair, threadIdx.x, rhs, nr);
 }
 
 // Coarsest level: x = B^{-1} b on the m listed unknowns (dense, FP64); one
-// warp per row.  Unlisted slots must be zero beforehand.
+// warp per row.  Unlisted slots of x are zero and stay so.  Up to 32 CR
+// unknowns a lane's part of the row and its slots are in registers before the
+// wait (the level's 512 unknowns by default: 16 entries a lane); larger
+// levels read the rest after it.  Four warps a block spread the rows over
+// the SMs (a row's 20 FP64 warp instructions take 0.15 us of an SM's pipe).
 template <typename T>
-__global__ void k_coarse_solve(int m, size_t S, const int *__restrict__ idx,
-                               const double *__restrict__ Binv,
-                               const T *__restrict__ b, T *__restrict__ x) {
-  pdl_entry();
-  b += (size_t)blockIdx.y * S;
-  x += (size_t)blockIdx.y * S;
+__global__ void __launch_bounds__(CS_THREADS)
+k_coarse_solve(int m, size_t S, const int *__restrict__ idx, const double *__restrict__ Binv,
+               const T *b, T *x) {
+  constexpr int CR = 16;
+  pdl_trigger();
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (warp >= m) return;
   const double *row = Binv + (size_t)warp * m;
+  double rv[CR];
+  int iv[CR];
+#pragma unroll
+  for (int k = 0; k < CR; ++k) {
+    const int j = lane + 32 * k;
+    const bool in = warp < m && j < m;
+    rv[k] = in ? row[j] : 0.0;
+    iv[k] = in ? idx[j] : -1;
+  }
+  const int out = warp < m ? idx[warp] : 0;
+  b += (size_t)blockIdx.y * S;
+  x += (size_t)blockIdx.y * S;
+  pdl_wait();
+  if (warp >= m) return;
+  T bv[CR];
+#pragma unroll
+  for (int k = 0; k < CR; ++k) bv[k] = iv[k] >= 0 ? b[iv[k]] : T(0);
   double acc = 0.0;
-  for (int j = lane; j < m; j += 32) acc += row[j] * (double)b[idx[j]];
+#pragma unroll
+  for (int k = 0; k < CR; ++k)
+    if (lane + 32 * k < m) acc += rv[k] * (double)bv[k];
+  for (int j = lane + 32 * CR; j < m; j += 32) acc += row[j] * (double)b[idx[j]];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0) x[idx[warp]] = (T)acc;
+  if (lane == 0) x[out] = (T)acc;
 }
 
 // ------------------------------------------------------------ launchers
+// Whether a level of nb bricks (times nk right-hand sides) takes the
+// quarter-brick kernels of spfd_slab.cu.  One CG iteration's launches, one
+// brick per block against quarter bricks (us, residual / sweep / restriction
+// onto the level): 48 bricks FP64 6.1 / 9.3 / 7.1 against 3.1 / 3.6 / 2.9,
+// FP32 3.6 / 3.3 / 4.4 against 1.6 / 1.9 / 1.8; 206 bricks FP64 9.9 / 11.7 /
+// 15.0 against 5.9 / 6.2 / 6.2, FP32 4.2 / 4.3 / 5.8 against 1.9 / 2.2 / 3.4;
+// 863 bricks FP64 17.8 / 18.0 / 21.2 against 15.8 / 20.6 / 22.9, FP32 8.6 /
+// 8.9 / 10.9 against 7.3 / 8.1 / 10.2; 4068 bricks FP64 66.9 / 71.4 against
+// 88.6 / 100, FP32 35.1 / 38.9 against 37.3 / 43.2 (there a brick's four
+// halos cost more than they save, and FP64 compaction works on fewer slots).
+template <typename T>
+constexpr bool slab_level(int nb, int nk, bool resid) {
+  return (long long)nb * nk <= (sizeof(T) == 4 || resid ? 1000 : 512);
+}
 template <typename T, typename C>
 void launch_residual7(const Grid &g, const C *gx, const T *diag, const T *x,
                       const T *b, T *r, cudaStream_t st, int nk, int order) {
@@ -618,6 +659,8 @@ template <typename T>
 void launch_residual27(const Grid &g, const T *stc, const T *x, const T *b,
                        T *r, cudaStream_t st, int nk, int order) {
   if (!g.nb) return;
+  if (order == 0 && slab_level<T>(g.nb, nk, true))
+    return launch_slab27<T>(g, stc, (const T *)nullptr, x, b, r, st, nk);
   if (order == 2) pdl(k_residual27<T, 2>, unit_grid(2, g.nb, nk), NT, st)(g, stc, x, b, r, nk);
   else if (order) pdl(k_residual27<T, 1>, unit_grid(1, g.nb, nk), NT, st)(g, stc, x, b, r, nk);
   else pdl(k_residual27<T, 0>, unit_grid(0, g.nb, nk), NT, st)(g, stc, x, b, r, nk);
@@ -680,7 +723,9 @@ void launch_jacobi27(const Grid &g, const T *stc, const T *wdinv, const T *xin,
                      const T *b, T *xout, cudaStream_t st, int nk, int order) {
   if (g.nb)
   {
-    if (order == 2)
+    if (order == 0 && slab_level<T>(g.nb, nk, false))
+      launch_slab27<T>(g, stc, wdinv, xin, b, xout, st, nk);
+    else if (order == 2)
       pdl(k_jacobi27<T, 2>, unit_grid(2, g.nb, nk), NT, st)(g, stc, wdinv, xin, b, xout, nk);
     else if (order)
       pdl(k_jacobi27<T, 1>, unit_grid(1, g.nb, nk), NT, st)(g, stc, wdinv, xin, b, xout, nk);
@@ -690,32 +735,29 @@ void launch_jacobi27(const Grid &g, const T *stc, const T *wdinv, const T *xin,
 }
 template <typename T>
 void launch_restrict(const Grid &gf, const Grid &gc, const T *P, const T *rf,
-                     T *bcoarse, cudaStream_t st, int nk, int order) {
-  if (gc.nb)
-  {
-    if (order == 2)
-      pdl(k_restrict<T, 2>, unit_grid(2, gc.nb, nk), NT, st)(gc, (size_t)gf.nb * BV, P, rf,
-                                                               bcoarse, nk);
-    else if (order)
-      pdl(k_restrict<T, 1>, unit_grid(1, gc.nb, nk), NT, st)(gc, (size_t)gf.nb * BV, P, rf,
-                                                               bcoarse, nk);
-    else
-      pdl(k_restrict<T, 0>, unit_grid(0, gc.nb, nk), NT, st)(gc, (size_t)gf.nb * BV, P, rf,
-                                                               bcoarse, nk);
-  }
+                     T *bcoarse, cudaStream_t st, int nk, int order, const T *wdinv, T *xc) {
+  if (!gc.nb) return;
+  const size_t Sf = (size_t)gf.nb * BV;
+  if (order == 2)
+    pdl(k_restrict<T, 2>, unit_grid(2, gc.nb, nk), NT, st)(gc, Sf, P, rf, bcoarse, nk, wdinv, xc);
+  else if (order)
+    pdl(k_restrict<T, 1>, unit_grid(1, gc.nb, nk), NT, st)(gc, Sf, P, rf, bcoarse, nk, wdinv, xc);
+  else if (slab_level<T>(gc.nb, nk, false))
+    launch_slab_restrict<T>(gc, Sf, P, wdinv, rf, bcoarse, xc, st, nk);
+  else
+    pdl(k_restrict<T, 0>, unit_grid(0, gc.nb, nk), NT, st)(gc, Sf, P, rf, bcoarse, nk, wdinv, xc);
 }
 template <typename T>
 void launch_prolong(const Grid &gf, const Grid &gc, const T *P, const T *ec,
                     T *ef, cudaStream_t st, int nk, int order) {
-  if (gf.nb)
-  {
-    if (order == 2)
-      pdl(k_prolong<T, 2>, unit_grid(2, (gf.nb + 1) / 2, nk), 128, st)(gf, gc, P, ec, ef, nk);
-    else if (order)
-      pdl(k_prolong<T, 1>, unit_grid(1, (gf.nb + 1) / 2, nk), 128, st)(gf, gc, P, ec, ef, nk);
-    else
-      pdl(k_prolong<T, 0>, unit_grid(0, (gf.nb + 1) / 2, nk), 128, st)(gf, gc, P, ec, ef, nk);
-  }
+  if (!gf.nb) return;
+  const int pairs = (gf.nb + 1) / 2;
+  if (order == 2)
+    pdl_early(k_prolong<T, 2>, unit_grid(2, pairs, nk), 128, st)(gf, gc, P, ec, ef, nk);
+  else if (order)
+    pdl_early(k_prolong<T, 1>, unit_grid(1, pairs, nk), 128, st)(gf, gc, P, ec, ef, nk);
+  else
+    pdl_early(k_prolong<T, 0>, unit_grid(0, pairs, nk), 128, st)(gf, gc, P, ec, ef, nk);
 }
 template <typename T, typename C>
 void launch_cheb7(const Grid &g, const C *gx, const T *diag, const T *wdinv, const T *xin,
@@ -746,8 +788,9 @@ template <typename T>
 void launch_coarse_solve(int m, size_t S, const int *idx, const double *Binv,
                          const T *b, T *x, cudaStream_t st, int nk) {
   if (m <= 0) return;
-  const int warps_per_block = 8;
-  pdl(k_coarse_solve<T>, dim3((m + warps_per_block - 1) / warps_per_block, nk), 32 * warps_per_block, st)(m, S, idx, Binv, b, x);
+  constexpr int WPB = CS_THREADS / 32;
+  pdl_early(k_coarse_solve<T>, dim3((m + WPB - 1) / WPB, nk), CS_THREADS, st)(m, S, idx, Binv, b,
+                                                                              x);
 }
 
 #define INST_T(T)                                                             \
@@ -762,7 +805,8 @@ void launch_coarse_solve(int m, size_t S, const int *idx, const double *Binv,
                                    const T *, const T *, T *, cudaStream_t,   \
                                    int, int);                                 \
   template void launch_restrict<T>(const Grid &, const Grid &, const T *,     \
-                                   const T *, T *, cudaStream_t, int, int);   \
+                                   const T *, T *, cudaStream_t, int, int,    \
+                                   const T *, T *);                           \
   template void launch_prolong<T>(const Grid &, const Grid &, const T *,      \
                                   const T *, T *, cudaStream_t, int, int);    \
   template void launch_coarse_solve<T>(int, size_t, const int *,              \

@@ -70,6 +70,26 @@ template <typename... P>
 inline PdlLaunch<P...> pdl(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t st) {
   return PdlLaunch<P...>{k, grid, block, st};
 }
+// pdl_early(kernel, grid, block, stream)(args...): the same launch for a
+// kernel that reads the operator before it waits.  Such a kernel begins with
+// pdl_trigger() and calls pdl_wait() once, in every thread.  Before the wait
+// it may read only what no kernel of a solve writes: the operators and
+// weights, activity bits and brick tables of the levels, which the build
+// finished and synchronised.  Vectors and Scalars are read and written after
+// it, through pointers without __restrict__, so that the compiler keeps
+// their loads behind the wait.  Triggering first is safe: the next kernel's
+// own wait holds it until this grid, which itself waits for its
+// predecessor, has completed.
+__device__ __forceinline__ void pdl_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... P>
+inline PdlLaunch<P...> pdl_early(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t st) {
+  return PdlLaunch<P...>{k, grid, block, st};
+}
 
 // Stencil offset index of (dx, dy, dz) in {-1,0,1}^3; 13 is the centre.
 __host__ __device__ __forceinline__ constexpr int sidx(int dx, int dy, int dz) {
@@ -248,14 +268,9 @@ __device__ __forceinline__ void act_stage(const Grid &g, int bk, ActList &al) {
   }
 }
 
-// Local slot (0..511) of the brick's n-th active slot, n < al.pre[16].
-__device__ __forceinline__ int act_slot(const ActList &al, int n) {
-  int j = 0;  // the last word whose prefix count is <= n (it holds slot n)
-#pragma unroll
-  for (int step = 8; step > 0; step >>= 1)
-    if (al.pre[j + step] <= n) j += step;
-  unsigned w = al.w[j];
-  int k = n - al.pre[j], pos = 0;  // the k-th set bit of w, by halving
+// Position of the k-th set bit of w (k < popcount), by halving.
+__device__ __forceinline__ int nth_bit(unsigned w, int k) {
+  int pos = 0;
 #pragma unroll
   for (int width = 16; width > 0; width >>= 1) {
     const unsigned lo = w & ((1u << width) - 1u);
@@ -268,8 +283,26 @@ __device__ __forceinline__ int act_slot(const ActList &al, int n) {
       w = lo;
     }
   }
-  return j * 32 + pos;
+  return pos;
 }
+
+// Local slot (0..511) of the brick's n-th active slot, n < al.pre[16].
+__device__ __forceinline__ int act_slot(const ActList &al, int n) {
+  int j = 0;  // the last word whose prefix count is <= n (it holds slot n)
+#pragma unroll
+  for (int step = 8; step > 0; step >>= 1)
+    if (al.pre[j + step] <= n) j += step;
+  return j * 32 + nth_bit(al.w[j], n - al.pre[j]);
+}
+
+// A thread's slot in a 27-point kernel: with compaction (FP64) thread n takes
+// the n-th active slot of its brick (or slab), else its own slot.  mine: the
+// thread computes the stencil at ts; idle: its own slot is inactive and gets
+// the zero-row result.
+struct SlotMap {
+  int ts;
+  bool mine, idle;
+};
 
 // Whether local slot t of the staged brick is active.
 __device__ __forceinline__ bool act_on(const ActList &al, int t) {
@@ -466,9 +499,22 @@ void launch_finish_rz(int n, const double *partials, double *scratch, Scalars *s
 template <typename T>
 void launch_jacobi27(const Grid &g, const T *stc, const T *wdinv, const T *xin,
                      const T *b, T *xout, cudaStream_t st, int nk = 1, int order = 0);
+// Restriction to the coarse level; with xc (single right-hand side) also
+// that level's first sweep from the zero guess, xc = wdinv bc (wdinv: the
+// coarse level's).
 template <typename T>
 void launch_restrict(const Grid &gf, const Grid &gc, const T *P, const T *rf,
-                     T *bc, cudaStream_t st, int nk = 1, int order = 0);
+                     T *bc, cudaStream_t st, int nk = 1, int order = 0,
+                     const T *wdinv = nullptr, T *xc = nullptr);
+// The quarter-brick kernels of small levels (spfd_slab.cu): the 27-point
+// weighted-Jacobi sweep (wdinv given) or residual (null), and the
+// restriction (as launch_restrict).
+template <typename T>
+void launch_slab27(const Grid &g, const T *st27, const T *wdinv, const T *x, const T *b, T *out,
+                   cudaStream_t st, int nk);
+template <typename T>
+void launch_slab_restrict(const Grid &gc, size_t Sf, const T *P, const T *wdinv, const T *rf,
+                          T *bc, T *xc, cudaStream_t st, int nk);
 template <typename T>
 void launch_prolong(const Grid &gf, const Grid &gc, const T *P, const T *ec,
                     T *ef, cudaStream_t st, int nk = 1, int order = 0);

@@ -54,17 +54,6 @@ __device__ __forceinline__ void ld_ints(const int *p, int (&c)[N]) {
   }
 }
 
-// Vector loads.  COH = false: plain loads (standalone kernels: what they
-// read was written by earlier launches).  COH = true: L2-only loads
-// (ld.global.cg), for a vector written by other blocks earlier in the same
-// launch (the fused coarse cycle), of which this SM's L1 may hold a stale
-// line.
-template <bool COH, typename T>
-__device__ __forceinline__ T ldv(const T *p) {
-  if constexpr (COH) return __ldcg(p);
-  else return *p;
-}
-
 // Neighbour brick ids of brick bk into shared memory (threads 0..26).
 __device__ __forceinline__ void load_nbr(const Grid &g, int bk, int *sn) {
   if (threadIdx.x < 27) sn[threadIdx.x] = g.nbr[(size_t)bk * 27 + threadIdx.x];
@@ -73,7 +62,7 @@ __device__ __forceinline__ void load_nbr(const Grid &g, int bk, int *sn) {
 // Brick + full halo of x (27-point stencils): the brick itself as 16-byte
 // vectors, the 488 halo values from the neighbour bricks one per thread
 // (planes tz = 0 and 9, then ty = 0 and 9, then tx = 0 and 9).
-template <typename T, bool COH = false>
+template <typename T>
 __device__ __forceinline__ void tile_full(T (*tl)[10][10], const T *__restrict__ x,
                                           int bk, const int *sn) {
   constexpr int VN = 16 / (int)sizeof(T), VPB = BV / VN;
@@ -81,9 +70,7 @@ __device__ __forceinline__ void tile_full(T (*tl)[10][10], const T *__restrict__
   if (t < VPB) {
     const int e0 = t * VN, lx = e0 & 7, ly = (e0 >> 3) & 7, lz = e0 >> 6;
     const T *p = x + (size_t)bk * BV + e0;
-    V16<T> v;
-    if constexpr (COH) *reinterpret_cast<uint4 *>(&v) = __ldcg(reinterpret_cast<const uint4 *>(p));
-    else v = ld16(p);
+    const V16<T> v = ld16(p);
     T *row = &tl[1 + lz][1 + ly][1 + lx];
 #pragma unroll
     for (int i = 0; i < VN; ++i) row[i] = v.v[i];
@@ -106,7 +93,7 @@ __device__ __forceinline__ void tile_full(T (*tl)[10][10], const T *__restrict__
     const int oz = tz == 0 ? -1 : (tz == 9 ? 1 : 0);
     const int nb = sn[sidx(ox, oy, oz)];
     tl[tz][ty][tx] = nb >= 0
-        ? ldv<COH>(&x[(size_t)nb * BV + (((tz - 1) & 7) * 8 + ((ty - 1) & 7)) * 8 + ((tx - 1) & 7)])
+        ? x[(size_t)nb * BV + (((tz - 1) & 7) * 8 + ((ty - 1) & 7)) * 8 + ((tx - 1) & 7)]
         : T(0);
   }
 }
