@@ -291,7 +291,7 @@ static ChebCoef cheb_coefficients(double hi, int k) {
 // is fused into the first sweep, using sum(r) left in each right-hand side's
 // Scalars by the preceding x/r update.
 template <typename T>
-T *vcycle(spfd_ctx *c, int l, T *bl, bool proj, int nk, bool rz, bool head) {
+T *vcycle(spfd_ctx *c, int l, T *bl, bool proj, int nk, int rz, bool head) {
   Level &lv = c->L[l];
   cudaStream_t st = c->stream;
   const int nl = (int)c->L.size();
@@ -408,17 +408,17 @@ T *vcycle(spfd_ctx *c, int l, T *bl, bool proj, int nk, bool rz, bool head) {
               launch_restrict<T>(lv.g, cl.g, cl.PP<T>(), lv.R<T>(), cl.B<T>(), st, nk,
                                  block_order(c, TF_RESTRICT, l), cl.WDINV<T>(),
                                  first ? cl.X<T>() : nullptr));
-  T *ec = vcycle<T>(c, l + 1, cl.B<T>(), false, nk, false, first);
+  T *ec = vcycle<T>(c, l + 1, cl.B<T>(), false, nk, -1, first);
   SPFD_LAUNCH(c, lvl_name(LVL_NAMES("prolong"), l), f32, 1,
               (27.0 / 8.0 + 2.0) * w * S + w * Sc, 7 * S,
               launch_prolong<T>(lv.g, cl.g, lv.PC<T>(), ec, cur, st, nk,
                                 block_order(c, TF_PROLONG, l)));
   for (int s = 0; s < c->opts.nu_post; ++s) {
-    if (rz && l == 0 && s + 1 == c->opts.nu_post)
-      SPFD_LAUNCH(c, "jacobi7_l0", f32, 1, (5 * w + 3 * wc) * S, 20 * S,
+    if (rz >= 0 && l == 0 && s + 1 == c->opts.nu_post)
+      SPFD_LAUNCH(c, "jacobi7_l0", f32, f32 ? 2 : 1, (5 * w + 3 * wc) * S, 20 * S,
                   (launch_jacobi7_rz<T, typename Prec<T>::C7>(
-                      lv.g, Prec<T>::gx(lv), lv.DIAG<T>(), wd, cur, bl, oth, c->partials,
-                      c->pstride, st, nk, block_order(c, TF_SMOOTH, l))));
+                      lv.g, Prec<T>::gx(lv), lv.DIAG<T>(), wd, cur, bl, oth, c->sc, rz,
+                      c->partials, c->pstride, st, nk, block_order(c, TF_SMOOTH, l))));
     else
       sweep(cur, oth);
     std::swap(cur, oth);
@@ -505,7 +505,8 @@ static spfd_status autotune_orders(spfd_ctx *c, int nk, std::vector<signed char>
       const T *opgx = sizeof(T) == 4 ? (const T *)lv.gx32 : (const T *)lv.gx;
       const T *opdiag = sizeof(T) == 4 ? (const T *)lv.diag32 : (const T *)lv.diag;
       TRY(pick(TF_APPLY, l, g.nb, false, [&](int o) {
-        launch_apply_dot<T>(g, opgx, opdiag, x, r, c->sc, c->partials, st, nk, c->pstride, o);
+        launch_apply_dot<T>(g, opgx, opdiag, x, r, c->sc, c->partials, c->pstride, st,
+                            nk, o);
       }));
     } else {
       TRY(pick(TF_SMOOTH, l, g.nb, true, [&](int o) {
@@ -598,20 +599,11 @@ spfd_status precondition_step(spfd_ctx *c, T *r, T *p, int first, int nk, bool h
   const double inv = c->ndof ? 1.0 / (double)c->ndof : 0.0;
   const double *csum = c->ncomp > 1 ? c->csum : nullptr;
   cudaStream_t st = c->stream;
-  // In FP32, r.z comes with the last level-0 sweep of the V-cycle when it
-  // has one: that sweep is HBM-bound, so the products and warp sums are free
-  // and a pass over r and z is saved.  The FP64 sweep is FP64-pipe-bound:
-  // its warp sums cost more than the separate pass (0.29 against 0.18 ms per
-  // sweep on the 2 mm body), so FP64 keeps k_dot_rz.
-  const bool fused = f32 && c->L.size() > 1 && c->opts.nu_post >= 1 &&
-                     c->opts.smoother == SPFD_SMOOTHER_JACOBI;
-  T *z = vcycle<T>(c, 0, r, true, nk, fused, head);
-  if (fused)
-    SPFD_LAUNCH(c, "finish_rz", false, 1, 16.0 * jacobi7_rz_partials<T>(nb) * nk, 0,
-                launch_finish_rz(jacobi7_rz_partials<T>(nb), c->partials,
-                                 c->partials + (size_t)16 * nb, c->sc, first, st, nk,
-                                 c->pstride, f32));
-  else
+  // r.z and the sum of z come with the last level-0 sweep of the V-cycle when
+  // it has one: both vectors are in its registers.
+  const bool fused = c->L.size() > 1 && c->opts.smoother == SPFD_SMOOTHER_JACOBI;
+  T *z = vcycle<T>(c, 0, r, true, nk, fused ? first : -1, head);
+  if (!fused)
     SPFD_LAUNCH(c, "dot_rz", f32, 1, (2 * w + 4) * S, 3 * S,
                 launch_dot_rz<T>(nb, r, z, c->comp, c->sc, c->partials, first, st, nk,
                                  c->pstride));
@@ -626,7 +618,7 @@ spfd_status precondition_step(spfd_ctx *c, T *r, T *p, int first, int nk, bool h
 template spfd_status precondition_step<double>(spfd_ctx *, double *, double *, int, int, bool);
 template spfd_status precondition_step<float>(spfd_ctx *, float *, float *, int, int, bool);
 template spfd_status project<double>(spfd_ctx *, double *, int, int);
-template double *vcycle<double>(spfd_ctx *, int, double *, bool, int, bool, bool);
+template double *vcycle<double>(spfd_ctx *, int, double *, bool, int, int, bool);
 
 struct PcgResult {
   int iters = 0;
@@ -726,13 +718,9 @@ static spfd_status pcg(spfd_ctx *c, T *x, T *r, T *p, T *q, const T *opgx,
       if (na == 0) break;
     }
     const double S = (double)S0 * na;
-    SPFD_LAUNCH(c, "apply_dot", f32, 1, (f32 ? 5 : 6) * w * S, (f32 ? 20 : 15) * S,
-                launch_apply_dot<T>(l0.g, opgx, opdiag, p, q, c->sc, c->partials, st, na,
-                                    c->pstride, block_order(c, TF_APPLY, 0)));
-    SPFD_LAUNCH(c, "finish_pq", false, 1, 8.0 * nb * na, nb * na,
-                launch_finish_pq(apply_dot_partials<T>(nb), c->partials,
-                                 c->partials + (size_t)16 * nb, c->sc, st, na, c->pstride,
-                                 f32));
+    SPFD_LAUNCH(c, "apply_dot", f32, f32 ? 2 : 1, (f32 ? 5 : 6) * w * S, (f32 ? 20 : 15) * S,
+                launch_apply_dot<T>(l0.g, opgx, opdiag, p, q, c->sc, c->partials, c->pstride, st,
+                                    na, block_order(c, TF_APPLY, 0)));
     SPFD_LAUNCH(c, "update_xr", f32, 1, 6 * w * S, 7 * S,
                 launch_update_xr<T>(nb, x, r, p, q, c->sc, c->partials, st, na, c->pstride));
     TRY(launch_check("CG update"));

@@ -487,11 +487,11 @@ spfd_status build_impl(spfd_ctx *c, const double *sigma) {
   clk.mark("level-0 tables");
   const size_t S0 = c->L[0].S;
   const int nb0 = c->L[0].g.nb;
-  // reduction scratch: the level-0 CG operator and the last smoothing sweep
-  // write at most 8 partials per brick (16 reserved), followed by the finishing reduction's block sums (152); the
-  // grid-stride reductions of every level write 2 values per block, on at
-  // most 608 blocks
-  c->pstride = 16 * (size_t)std::max(nb0, 1) + 2048;
+  // reduction scratch: the level-0 FP32 row kernels write up to two pairs (of
+  // 8 bytes) for each of a brick's four warps; the FP64 kernels that walk the
+  // bricks and the grid-stride reductions 2 values per block on at most 760
+  // blocks
+  c->pstride = 8 * (size_t)nb0 + 2048;
   TRY(dalloc(c, &c->partials, c->pstride));
   int *parent = nullptr, *counts = nullptr, *offsets = nullptr;
   int *comp_hcnt = nullptr, *comp_hstat = nullptr;

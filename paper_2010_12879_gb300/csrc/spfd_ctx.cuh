@@ -308,9 +308,10 @@ inline int block_order(const spfd_ctx *c, int fam, int l) {
 template <typename T>
 spfd_status project(spfd_ctx *c, T *v, int nk = 1, int j0 = 0);
 // V-cycle on level l for nk right-hand sides; returns the corrections.
-// head: the level-0 cycle's first sweep already ran (vcycle_head).
+// rz >= 0 (level 0): the last sweep also forms r.z and beta (rz = 1: on the
+// first iteration, beta = 0).  head: the cycle's first sweep already ran.
 template <typename T>
-T *vcycle(spfd_ctx *c, int l, T *bl, bool proj, int nk, bool rz = false, bool head = false);
+T *vcycle(spfd_ctx *c, int l, T *bl, bool proj, int nk, int rz = -1, bool head = false);
 // z = M r, r.z, beta and p = z + beta p for the first nk right-hand sides.
 template <typename T>
 spfd_status precondition_step(spfd_ctx *c, T *r, T *p, int first, int nk, bool head = false);

@@ -10,6 +10,7 @@
 // per thread without shared memory on level 0, one node per thread with a shared tile on the
 // 27-point levels (spfd_tile.cuh).
 #include "spfd_internal.cuh"
+#include "spfd_reduce.cuh"
 #include "spfd_tile.cuh"
 
 namespace spfd {
@@ -41,16 +42,11 @@ k_residual7(Grid g, const C *__restrict__ gx, const T *__restrict__ diag,
   stqn<T, N>(r + s0, rv);
 }
 
-// RZ: the last sweep of the V-cycle on level 0, where b is the CG residual r
-// and xout the preconditioned z: each warp also writes its parts of r.z and
-// of the sum of z over the unknowns (w > 0) to partials[2 (brick warp) + {0,1}]
-// (right-hand side rhs at rhs * pstride), which launch_finish_rz adds.
-template <typename T, typename C, int ORD, bool RZ = false>
+template <typename T, typename C, int ORD>
 __global__ void __launch_bounds__(BV / row_n_jacobi<T>(), row_min_blocks_jacobi<T>())
 k_jacobi7(Grid g, const C *__restrict__ gx, const T *__restrict__ diag,
           const T *__restrict__ wdinv, const T *__restrict__ xin,
-          const T *__restrict__ b, T *__restrict__ xout, int nk,
-          double *__restrict__ partials = nullptr, size_t pstride = 0) {
+          const T *__restrict__ b, T *__restrict__ xout, int nk) {
   pdl_entry();
   constexpr int N = row_n_jacobi<T>();
   int bk, rhs;
@@ -65,20 +61,61 @@ k_jacobi7(Grid g, const C *__restrict__ gx, const T *__restrict__ diag,
 #pragma unroll
   for (int i = 0; i < N; ++i) xc.v[i] += wv.v[i] * rv.v[i];
   stqn<T, N>(xout + s0, xc);
-  if constexpr (RZ) {
-    T rz[N], zs[N];
+}
+
+// The last sweep of the V-cycle on level 0, where b is the CG residual r and
+// xout the preconditioned z: also sums r.z and z (z is zero at slots that are
+// not unknowns) and sets beta and the mean of z, in FP64 by blocks that walk
+// the bricks (walk_units), in FP32 by pairs and k_finish_pairs (see k_apply_dot).  2 mm
+// body, with the r.z pass or finishing kernel it replaces: FP64 157 + 55 ->
+// 204 us (two more FP64 operations a node on the pipe that bounds the sweep,
+// against a pass over r and z).
+template <typename T, typename C, int ORD>
+__global__ void __launch_bounds__(BV / row_n_jacobi<T>(), row_min_blocks_jacobi<T>())
+k_jacobi7_rz(Grid g, const C *__restrict__ gx, const T *__restrict__ diag,
+             const T *__restrict__ wdinv, const T *__restrict__ xin,
+             const T *__restrict__ b, T *__restrict__ xout, int nk, int units,
+             Scalars *sc, int first, double *partials, size_t pstride) {
+  pdl_entry();
+  constexpr int N = row_n_jacobi<T>(), THREADS = BV / N;
+  int unit, rhs;
+  unit_rhs<ORD>(nk, unit, rhs);
+  const int t = threadIdx.x;
+  const size_t S = (size_t)g.nb * BV, off = (size_t)rhs * S;
+  xin += off; b += off; xout += off;
+  sc += rhs;
+  partials += (size_t)rhs * pstride;
+  auto sweep = [&](int bk, Qv<T, N> &bv, Qv<T, N> &xc) {
+    const size_t s0 = row_slot<N>(bk, t);
+    bv = ldqn<T, T, N>(b + s0);
+    const Qv<T, N> wv = ldqn<T, T, N>(wdinv + s0);
+    Qv<T, N> rv;
+    apply7_row<T, C, true, N>(g, gx, diag, xin, S, bk, t, bv, xc, rv);
+#pragma unroll
+    for (int i = 0; i < N; ++i) xc.v[i] += wv.v[i] * rv.v[i];
+    stqn<T, N>(xout + s0, xc);
+  };
+  Qv<T, N> bv, xc;
+  if constexpr (sizeof(T) == 4) {
+    sweep(unit, bv, xc);
+    float v[2][N];
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      rz[i] = bv.v[i] * xc.v[i];
-      zs[i] = weight_pos(wv.v[i]) ? xc.v[i] : (T)0;
+      v[0][i] = bv.v[i] * xc.v[i];
+      v[1][i] = xc.v[i];
     }
-    const WarpSum<T> prz = warp_total<T, N>(rz), pzs = warp_total<T, N>(zs);
-    if ((t & 31) == 0) {
-      double *pp = partials + (size_t)rhs * pstride +
-                   2 * ((size_t)bk * (BV / N / 32) + (t >> 5));
-      prz.put(pp);
-      pzs.put(pp + 1);
+    warp_pairs<2, N>(v, unit * (THREADS / 32) + (t >> 5), partials);
+  } else {
+    double v[2] = {0.0, 0.0}, tot[2];
+    for (int bk = unit; bk < g.nb; bk += units) {
+      sweep(bk, bv, xc);
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        v[0] += bv.v[i] * xc.v[i];
+        v[1] += xc.v[i];
+      }
     }
+    if (grid_sum<2, THREADS>(v, partials, &sc->ticket[2], tot, unit, units)) set_rz(sc, tot, first);
   }
 }
 
@@ -691,32 +728,28 @@ void launch_jacobi_first_proj(const Grid &g, const T *wdinv, T *b, T *x,
 }
 template <typename T, typename C>
 void launch_jacobi7_rz(const Grid &g, const C *gx, const T *diag, const T *wdinv,
-                       const T *xin, const T *b, T *xout, double *partials, size_t pstride,
-                       cudaStream_t st, int nk, int order) {
+                       const T *xin, const T *b, T *xout, Scalars *sc, int first,
+                       double *partials, size_t pstride, cudaStream_t st, int nk, int order) {
   if (!g.nb) return;
+  const int units = sizeof(T) == 4 ? g.nb : walk_units(g.nb, row_min_blocks_jacobi<T>());
   if (order)
-    pdl(k_jacobi7<T, C, 1, true>, unit_grid(1, g.nb, nk), BV / row_n_jacobi<T>(), st)(
-        g, gx, diag, wdinv, xin, b, xout, nk, partials, pstride);
+    pdl(k_jacobi7_rz<T, C, 1>, unit_grid(1, units, nk), BV / row_n_jacobi<T>(), st)(
+        g, gx, diag, wdinv, xin, b, xout, nk, units, sc, first, partials, pstride);
   else
-    pdl(k_jacobi7<T, C, 0, true>, unit_grid(0, g.nb, nk), BV / row_n_jacobi<T>(), st)(
-        g, gx, diag, wdinv, xin, b, xout, nk, partials, pstride);
+    pdl(k_jacobi7_rz<T, C, 0>, unit_grid(0, units, nk), BV / row_n_jacobi<T>(), st)(
+        g, gx, diag, wdinv, xin, b, xout, nk, units, sc, first, partials, pstride);
+  if (sizeof(T) == 4) launch_finish_pairs(true, g.nb, partials, sc, first, pstride, st, nk);
 }
-template <typename T>
-int jacobi7_rz_partials(int nb) { return nb * (BV / row_n_jacobi<T>() / 32); }
-template int jacobi7_rz_partials<double>(int);
-template int jacobi7_rz_partials<float>(int);
 template <typename T, typename C>
 void launch_jacobi7(const Grid &g, const C *gx, const T *diag, const T *wdinv,
                     const T *xin, const T *b, T *xout, cudaStream_t st, int nk, int order) {
-  if (g.nb)
-  {
-    if (order)
-      pdl(k_jacobi7<T, C, 1>, unit_grid(1, g.nb, nk), BV / row_n_jacobi<T>(), st)(
-          g, gx, diag, wdinv, xin, b, xout, nk, nullptr, (size_t)0);
-    else
-      pdl(k_jacobi7<T, C, 0>, unit_grid(0, g.nb, nk), BV / row_n_jacobi<T>(), st)(
-          g, gx, diag, wdinv, xin, b, xout, nk, nullptr, (size_t)0);
-  }
+  if (!g.nb) return;
+  if (order)
+    pdl(k_jacobi7<T, C, 1>, unit_grid(1, g.nb, nk), BV / row_n_jacobi<T>(), st)(
+        g, gx, diag, wdinv, xin, b, xout, nk);
+  else
+    pdl(k_jacobi7<T, C, 0>, unit_grid(0, g.nb, nk), BV / row_n_jacobi<T>(), st)(
+        g, gx, diag, wdinv, xin, b, xout, nk);
 }
 template <typename T>
 void launch_jacobi27(const Grid &g, const T *stc, const T *wdinv, const T *xin,
@@ -822,8 +855,8 @@ INST_T(float)
 #define INST_TC(T, C)                                                         \
   template void launch_jacobi7_rz<T, C>(const Grid &, const C *, const T *,   \
                                         const T *, const T *, const T *, T *, \
-                                        double *, size_t, cudaStream_t, int,  \
-                                        int);                                 \
+                                        Scalars *, int, double *, size_t,     \
+                                        cudaStream_t, int, int);              \
   template void launch_residual7<T, C>(const Grid &, const C *, const T *,    \
                                        const T *, const T *, T *,             \
                                        cudaStream_t, int, int);               \

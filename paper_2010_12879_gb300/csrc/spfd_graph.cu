@@ -361,10 +361,7 @@ spfd_status capture_solve_fp64(spfd_ctx *c, GraphCtl *ctl, const double *a, doub
     cudaStream_t s1 = body[0];
     SPFD_LAUNCH(c, "apply_dot", false, 1, 6 * 8 * S, 15 * S,
                 launch_apply_dot<double>(l0.g, l0.gx, l0.diag, c->pk, c->qk, c->sc,
-                                         c->partials, s1, 1, c->pstride));
-    SPFD_LAUNCH(c, "finish_pq", false, 1, 8.0 * nb, nb,
-                launch_finish_pq(apply_dot_partials<double>(nb), c->partials,
-                                 c->partials + (size_t)16 * nb, c->sc, s1, 1, c->pstride));
+                                         c->partials, c->pstride, s1));
     SPFD_LAUNCH(c, "update_xr", false, 1, 6 * 8 * S, 7 * S,
                 launch_update_xr<double>(nb, c->xk, c->rk, c->pk, c->qk, c->sc, c->partials,
                                          s1, 1, c->pstride));
@@ -485,11 +482,7 @@ spfd_status capture_solve_mixed(spfd_ctx *c, GraphCtl *ctl, const double *a, dou
         c->stream = s3;
         SPFD_LAUNCH(c, "apply_dot", true, 1, 5 * 4 * S, 20 * S,
                     launch_apply_dot<float>(l0.g, l0.gx32, l0.diag32, c->pk32, c->qk32, c->sc,
-                                            c->partials, s3, 1, c->pstride));
-        SPFD_LAUNCH(c, "finish_pq", false, 1, 8.0 * nb, nb,
-                    launch_finish_pq(apply_dot_partials<float>(nb), c->partials,
-                                     c->partials + (size_t)16 * nb, c->sc, s3, 1, c->pstride,
-                                     true));
+                                            c->partials, c->pstride, s3));
         SPFD_LAUNCH(c, "update_xr", true, 1, 6 * 4 * S, 7 * S,
                     launch_update_xr<float>(nb, c->dk32, c->rk32, c->pk32, c->qk32, c->sc,
                                             c->partials, s3, 1, c->pstride));

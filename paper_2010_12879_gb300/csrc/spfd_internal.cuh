@@ -146,6 +146,16 @@ inline dim3 unit_grid(int order, int units, int nk) {
   if (order == 2) return dim3((unsigned)units, (unsigned)((nk + RHS_TILE - 1) / RHS_TILE));
   return order ? dim3((unsigned)units * (unsigned)nk) : dim3((unsigned)units, (unsigned)nk);
 }
+// Blocks of a kernel that walks the bricks (block u takes bricks u, u + units,
+// ...): at most as many as are resident at once on 152 SMs with per_sm blocks
+// each, and so many that all walk equally far (3412 bricks over 1368 resident
+// blocks: 1138 blocks of three each instead of 1368 of which half do two).
+// It depends on the level alone, so that the sums such a kernel forms do not
+// depend on the number of right-hand sides.
+inline int walk_units(int nb, int per_sm) {
+  const int res = 152 * per_sm, rounds = (nb + res - 1) / res;
+  return (nb + rounds - 1) / rounds;
+}
 // Order 1 is available while units * nk fits a one-dimensional grid.
 inline bool order1_fits(int units, int nk) {
   return (long long)units * nk <= 2147483647LL;
@@ -484,18 +494,12 @@ void launch_jacobi7(const Grid &g, const C *gx, const T *diag, const T *wdinv,
                     const T *xin, const T *b, T *xout, cudaStream_t st, int nk = 1,
                     int order = 0);
 // The same sweep as the last one of the V-cycle on level 0 (b = r, xout =
-// z): also writes 2 partials (r.z, sum of z over the unknowns) per warp,
-// jacobi7_rz_partials(nb) pairs per right-hand side, for launch_finish_rz.
+// z), with r.z, beta and the mean of z as launch_dot_rz forms them.
 template <typename T, typename C>
 void launch_jacobi7_rz(const Grid &g, const C *gx, const T *diag, const T *wdinv,
-                       const T *xin, const T *b, T *xout, double *partials, size_t pstride,
-                       cudaStream_t st, int nk = 1, int order = 0);
-template <typename T> int jacobi7_rz_partials(int nb);
-// Adds n pairs of partials (scratch: at least 304 doubles, not overlapping)
-// and sets rz, beta, zsum and zmean as launch_dot_rz does.
-// pairs: the partials are FP32 (hi, lo) pairs (FP32 producers).
-void launch_finish_rz(int n, const double *partials, double *scratch, Scalars *sc, int first,
-                      cudaStream_t st, int nk = 1, size_t pstride = 0, bool pairs = false);
+                       const T *xin, const T *b, T *xout, Scalars *sc, int first,
+                       double *partials, size_t pstride, cudaStream_t st, int nk = 1,
+                       int order = 0);
 template <typename T>
 void launch_jacobi27(const Grid &g, const T *stc, const T *wdinv, const T *xin,
                      const T *b, T *xout, cudaStream_t st, int nk = 1, int order = 0);
@@ -543,17 +547,15 @@ void launch_coarse_solve(int m, size_t S, const int *idx, const double *Binv,
 // launch (blockIdx.y): level-0 vectors are nk blocks of S0 values, sc points
 // at nk consecutive Scalars, partials at nk regions pstride apart, csum at nk
 // blocks of ncomp sums; edge and node-grid arrays are nk blocks of 3 NN / NN.
+// q = A p, p.q and alpha = rz / p.q (FP32: two launches).
 template <typename T>
 void launch_apply_dot(const Grid &g, const T *gx, const T *diag, const T *p,
-                      T *q, Scalars *sc, double *partials, cudaStream_t st, int nk = 1,
-                      size_t pstride = 0, int order = 0);
-// Number of partial sums launch_apply_dot writes for nb bricks (one per warp,
-// 8 per brick in FP64, 4 in FP32, where each is an FP32 (hi, lo) pair in its
-// 8-byte slot); launch_finish_pq adds n of them (scratch: at least 152
-// doubles, not overlapping; pairs for FP32 partials) and sets alpha = rz / pq.
-template <typename T> int apply_dot_partials(int nb);
-void launch_finish_pq(int n, const double *partials, double *scratch, Scalars *sc,
-                      cudaStream_t st, int nk = 1, size_t pstride = 0, bool pairs = false);
+                      T *q, Scalars *sc, double *partials, size_t pstride, cudaStream_t st,
+                      int nk = 1, int order = 0);
+// Adds the FP32 pairs of the level-0 row kernels, four warps per brick: p.q
+// and alpha, or (rz) r.z, beta and the mean of z.
+void launch_finish_pairs(bool rz, int nb, const double *pairs, Scalars *sc, int first,
+                         size_t pstride, cudaStream_t st, int nk);
 // x += alpha p, r -= alpha q, r.r, sum r; right-hand sides whose Scalars are
 // frozen are left as they are.
 template <typename T>

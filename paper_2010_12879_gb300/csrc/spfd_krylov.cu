@@ -13,242 +13,129 @@
 // and blocks.
 #include <algorithm>
 
+#include <cooperative_groups.h>
+
 #include "spfd_internal.cuh"
+#include "spfd_reduce.cuh"
 #include "spfd_tile.cuh"
 
 namespace spfd {
-
-// ------------------------------------------------------------ accumulators
-// Per-thread running sum: FP64 for double kernels, compensated FP32 for float
-// kernels (about FP64 accuracy over the few dozen terms a thread adds).
-template <typename T> struct Acc;
-template <> struct Acc<double> {
-  double s = 0.0;
-  __device__ __forceinline__ void add(double v) { s += v; }
-  __device__ __forceinline__ double get() const { return s; }
-};
-template <> struct Acc<float> {
-  float s = 0.f, c = 0.f;
-  __device__ __forceinline__ void add(float v) {
-    const float y = v - c;
-    const float t = s + y;
-    c = (t - s) - y;
-    s = t;
-  }
-  __device__ __forceinline__ double get() const { return (double)s - (double)c; }
-};
-
-// ------------------------------------------------------------ reductions
-// Block sums of the threads' NV FP64 values, left in warp 0 (every lane),
-// for blocks of at most NT threads.  The values pass through shared memory
-// and warp 0 adds them (lane l the values of threads l, l + 32, ..., then a
-// butterfly): NV * (warps + 4) FP64 warp instructions per block, against
-// 5 NV per warp plus 5 NV for a butterfly in every warp, on GB300's narrow
-// FP64 pipe.
-template <int NV>
-__device__ __forceinline__ void block_sum(double (&v)[NV]) {
-  __shared__ double sm[NV][NT];
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const int nw = (blockDim.x + 31) >> 5;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) sm[k][t] = v[k];
-  __syncthreads();
-  if (w == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double a = sm[k][lane];
-      for (int i = 1; i < nw; ++i) a += sm[k][lane + 32 * i];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-      v[k] = a;
-    }
-  }
-  __syncthreads();
-}
-
-// The tail of the grid reductions, once thread 0 has written this block's NV
-// partials: a ticket finds the last block, which adds every block's partials
-// in a fixed order.  Returns true in thread 0 of the last block, with tot[] =
-// grid totals.
-template <int NV>
-__device__ bool grid_finish(double *partials, unsigned *ticket, double (&tot)[NV]) {
-  __shared__ bool last;
-  if (threadIdx.x == 0) {
-    __threadfence();
-    unsigned prev = atomicAdd(ticket, 1u);
-    last = prev == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!last) return false;
-  __threadfence();
-  double a[NV];
-#pragma unroll
-  for (int k = 0; k < NV; ++k) a[k] = 0.0;
-  for (unsigned i = threadIdx.x; i < gridDim.x; i += blockDim.x)
-#pragma unroll
-    for (int k = 0; k < NV; ++k) a[k] += __ldcg(&partials[(size_t)i * NV + k]);
-  block_sum<NV>(a);
-  if (threadIdx.x != 0) return false;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) tot[k] = a[k];
-  *ticket = 0u;
-  return true;
-}
-
-template <int NV>
-__device__ bool grid_sum(double (&v)[NV], double *partials, unsigned *ticket,
-                         double (&tot)[NV]) {
-  block_sum<NV>(v);
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int k = 0; k < NV; ++k) partials[(size_t)blockIdx.x * NV + k] = v[k];
-  return grid_finish<NV>(partials, ticket, tot);
-}
-
-// hi + lo += oh + ol with the rounding error of the high parts kept (TwoSum).
-__device__ __forceinline__ void two_sum_add(float &hi, float &lo, float oh, float ol) {
-  const float s = hi + oh, bb = s - hi;
-  const float e = (hi - (s - bb)) + (oh - bb);
-  hi = s;
-  lo = lo + ol + e;
-}
-
-// grid_sum for per-thread FP32 pairs (value hi + lo): the warps and the block
-// add them as TwoSum pairs in FP32, and only the block's total is widened to
-// FP64 (in thread 0).  An FP64 conversion or addition takes a 16-clock slot
-// of GB300's narrow FP64 pipe for its warp whatever its lane mask, so
-// widening in every thread put an FP64 tail of several microseconds at the
-// end of the FP32 reduction kernels.
-template <int NV>
-__device__ bool grid_sum_f32(float (&hi)[NV], float (&lo)[NV], double *partials,
-                             unsigned *ticket, double (&tot)[NV]) {
-  __shared__ float sh[32][NV], sl[32][NV];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int nw = (blockDim.x + 31) >> 5;
-#pragma unroll
-  for (int k = 0; k < NV; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-      two_sum_add(hi[k], lo[k], __shfl_xor_sync(0xffffffffu, hi[k], o),
-                  __shfl_xor_sync(0xffffffffu, lo[k], o));
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      sh[w][k] = hi[k];
-      sl[w][k] = lo[k];
-    }
-  __syncthreads();
-  if (w == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      float h = lane < nw ? sh[lane][k] : 0.f, l = lane < nw ? sl[lane][k] : 0.f;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1)
-        two_sum_add(h, l, __shfl_xor_sync(0xffffffffu, h, o), __shfl_xor_sync(0xffffffffu, l, o));
-      if (lane == 0) partials[(size_t)blockIdx.x * NV + k] = (double)h + (double)l;
-    }
-  }
-  return grid_finish<NV>(partials, ticket, tot);
-}
-
-// grid_sum of per-thread accumulators: FP64 sums directly, compensated FP32
-// sums (value s - c) as FP32 pairs.
-template <typename T, int NV>
-__device__ bool grid_sum_acc(const Acc<T> (&a)[NV], double *partials, unsigned *ticket,
-                             double (&tot)[NV]) {
-  if constexpr (sizeof(T) == 8) {
-    double v[NV];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) v[k] = a[k].s;
-    return grid_sum<NV>(v, partials, ticket, tot);
-  } else {
-    float h[NV], l[NV];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      h[k] = a[k].s;
-      l[k] = -a[k].c;
-    }
-    return grid_sum_f32<NV>(h, l, partials, ticket, tot);
-  }
-}
 
 // Grid-stride reduction kernels use at most RED_GRID blocks, so the ticket
 // sees few same-address atomics.
 constexpr int RED_GRID = 608;  // 4 resident 512-thread blocks on each of 152 SMs
 
 // ------------------------------------------------------------ CG operator
-// q = A p on one brick per block (row mapping, four nodes per thread); each
-// warp writes its part of p.q, and k_finish_pq adds them.  A right-hand side
-// that has converged (frozen) gets q = 0 and p.q = 0 without its operator
-// work.  (Written as that warp-uniform branch, the FP64 operator also
-// measured 8 % faster than the unconditional form, 193 against 211 us per
-// launch on the 2 mm body.)
+// q = A p and p.q (row mapping, four nodes per thread), then alpha = rz / p.q.
+// FP64: the blocks are resident all at once and walk the bricks (walk_units),
+// so that p.q is summed over a thread's bricks and reduced once per block:
+// with one brick per block each warp spent five of its 37 FP64 instructions a
+// brick on its butterfly, on the pipe that bounds this kernel, and 89,000
+// partial sums (2 mm body) took a kernel of their own to add: 187 + 6 us
+// together, 171 us now.  (Blocks that take 2, 4 or 8 consecutive bricks before
+// they step, for the sake of the x-faces in L1, measured 177, 194 and 195 us.)
+// FP32 is bound by memory, where walking costs more registers than it saves
+// (53 us against 47): one brick per block, a pair per warp, and
+// k_finish_pairs.
+// A right-hand side that has converged (frozen) is left alone.
 template <typename T, int ORD>
 __global__ void __launch_bounds__(BV / row_n_apply<T>(), row_min_blocks_apply<T>())
 k_apply_dot(Grid g, const T *__restrict__ gx, const T *__restrict__ diag,
-            const T *__restrict__ p, T *__restrict__ q, const Scalars *sc,
-            double *partials, size_t pstride, int nk) {
+            const T *__restrict__ p, T *__restrict__ q, Scalars *sc,
+            double *partials, size_t pstride, int nk, int units) {
   pdl_entry();
-  constexpr int N = row_n_apply<T>(), NW = BV / N / 32;
-  int bk, rhs;
-  unit_rhs<ORD>(nk, bk, rhs);
+  constexpr int N = row_n_apply<T>(), THREADS = BV / N;
+  int unit, rhs;
+  unit_rhs<ORD>(nk, unit, rhs);
+  sc += rhs;
+  if (sc->frozen) return;
   const int t = threadIdx.x;
-  const size_t S = (size_t)g.nb * BV, s0 = row_slot<N>(bk, t);
+  const size_t S = (size_t)g.nb * BV;
   p += (size_t)rhs * S;
   q += (size_t)rhs * S;
   partials += (size_t)rhs * pstride;
   Qv<T, N> pc, qv;
-  if (__any_sync(0xffffffffu, !sc[rhs].frozen)) {
-    apply7_row<T, T, false, N, sizeof(T) == 8>(g, gx, diag, p, S, bk, t, zqn<T, N>(), pc, qv);
-  } else {
-    pc = zqn<T, N>();
-    qv = zqn<T, N>();
-  }
-  stqn<T, N>(q + s0, qv);
   if constexpr (sizeof(T) == 4) {
-    // FP32 products summed without rounding error in (hi, lo) pairs
-    // (TwoSum) over the thread's nodes and the warp, rounded to FP64 in the
-    // storing lane only
-    float pq[N];
+    apply7_row<T, T, false, N, false>(g, gx, diag, p, S, unit, t, zqn<T, N>(), pc, qv);
+    stqn<T, N>(q + row_slot<N>(unit, t), qv);
+    float pq[1][N];
 #pragma unroll
-    for (int i = 0; i < N; ++i) pq[i] = pc.v[i] * qv.v[i];
-    const WarpSum<float> part = warp_total<float, N>(pq);
-    if ((t & 31) == 0) part.put(&partials[(size_t)bk * NW + (t >> 5)]);
+    for (int i = 0; i < N; ++i) pq[0][i] = pc.v[i] * qv.v[i];
+    warp_pairs<1, N>(pq, unit * (THREADS / 32) + (t >> 5), partials);
   } else {
-    double a = pc.v[0] * qv.v[0];
+    double v[1] = {0.0}, tot[1];
+    for (int bk = unit; bk < g.nb; bk += units) {
+      apply7_row<T, T, false, N, true>(g, gx, diag, p, S, bk, t, zqn<T, N>(), pc, qv);
+      stqn<T, N>(q + row_slot<N>(bk, t), qv);
 #pragma unroll
-    for (int i = 1; i < N; ++i) a += pc.v[i] * qv.v[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if ((t & 31) == 0) partials[(size_t)bk * NW + (t >> 5)] = a;
+      for (int i = 0; i < N; ++i) v[0] += pc.v[i] * qv.v[i];
+    }
+    if (grid_sum<1, THREADS>(v, partials, &sc->ticket[6], tot, unit, units)) set_pq(sc, tot[0]);
   }
 }
 
-// Number of partials k_apply_dot writes for nb bricks.
-template <typename T>
-int apply_dot_partials(int nb) { return nb * (BV / row_n_apply<T>() / 32); }
-
-// pq = sum of the n partials of k_apply_dot (blocks add contiguous chunks,
-// the last block adds the block sums, fixed order); alpha = rz / pq.
-// scratch must not overlap the partials.
-template <bool PAIRS>
-__global__ void __launch_bounds__(NT)
-k_finish_pq(const double *__restrict__ partials, int n, double *scratch, Scalars *sc,
-            size_t pstride) {
+// The n (times NV) pairs of an FP32 row kernel added, and the scalars set: NV =
+// 1 p.q and alpha, NV = 2 r.z, beta and the mean of z.  One cluster of eight
+// blocks per right-hand side: the threads add pairs without rounding error,
+// each block's total is widened to FP64 and passed to the first block through
+// its shared memory.  A grid with a ticket (fence, atomic, second round
+// through L2) took 7.4 us for 89,000 pairs and 12.3 us for twice as many.
+constexpr int FP_CLUSTER = 8, FP_THREADS = 1024;
+template <int NV>
+__global__ void __cluster_dims__(FP_CLUSTER, 1, 1) __launch_bounds__(FP_THREADS)
+k_finish_pairs(const double *__restrict__ pairs, int n, Scalars *sc, int first,
+               size_t pstride) {
   pdl_entry();
-  partials += (size_t)blockIdx.y * pstride;
-  scratch += (size_t)blockIdx.y * pstride;
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  __shared__ double all[FP_CLUSTER][NV];
+  __shared__ float sh[32][NV], sl[32][NV];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const float2 *pp = reinterpret_cast<const float2 *>(pairs + (size_t)blockIdx.y * pstride);
   sc += blockIdx.y;
-  double a = 0.0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    a += pair_at<PAIRS>(partials, i);
-  double v[1] = {a};
-  double tot[1];
-  if (grid_sum<1>(v, scratch, &sc->ticket[6], tot)) {
-    sc->pq = tot[0];
-    const double al = tot[0] > 0.0 ? sc->rz / tot[0] : 0.0;
-    sc->alpha = al;
-    sc->alpha_f = (float)al;
+  if (NV == 1 && sc->frozen) return;  // the whole cluster: its operator wrote nothing
+  float hi[NV], lo[NV];
+#pragma unroll
+  for (int k = 0; k < NV; ++k) hi[k] = lo[k] = 0.f;
+#pragma unroll 4
+  for (int i = blockIdx.x * FP_THREADS + t; i < n; i += FP_CLUSTER * FP_THREADS)
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      const float2 q = pp[(size_t)NV * i + k];
+      two_sum_add(hi[k], lo[k], q.x, q.y);
+    }
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      two_sum_add(hi[k], lo[k], __shfl_xor_sync(0xffffffffu, hi[k], o),
+                  __shfl_xor_sync(0xffffffffu, lo[k], o));
+    if (lane == 0) {
+      sh[w][k] = hi[k];
+      sl[w][k] = lo[k];
+    }
+  }
+  __syncthreads();
+  if (w == 0) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      float h = sh[lane][k], l = sl[lane][k];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+        two_sum_add(h, l, __shfl_xor_sync(0xffffffffu, h, o), __shfl_xor_sync(0xffffffffu, l, o));
+      if (lane == 0)
+        cl.map_shared_rank(&all[0][0], 0)[NV * cl.block_rank() + k] = (double)h + (double)l;
+    }
+  }
+  cl.sync();
+  if (cl.block_rank() == 0 && t == 0) {
+    double tot[2] = {0.0, 0.0};
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+#pragma unroll
+      for (int b = 0; b < FP_CLUSTER; ++b) tot[k] += all[b][k];
+    if constexpr (NV == 1) set_pq(sc, tot[0]);
+    else set_rz(sc, tot, first);
   }
 }
 
@@ -289,7 +176,7 @@ k_update_xr(int nb, T *__restrict__ x, T *__restrict__ r,
   }
   const Acc<T> v[2] = {rr, rs_sum};
   double tot[2];
-  if (grid_sum_acc<T, 2>(v, partials, &sc->ticket[1], tot)) {
+  if (grid_sum_acc<T, 2>(v, partials, &sc->ticket[1], tot, blockIdx.x, gridDim.x)) {
     sc->rr = tot[0];
     sc->rsum = tot[1];
     sc->rmean = tot[1] * sc->inv_ndof;
@@ -299,22 +186,6 @@ k_update_xr(int nb, T *__restrict__ x, T *__restrict__ r,
 
 // rz = r.z (new), beta = rz / rz_old, zsum = sum of z over the unknowns and
 // zmean = zsum / n.
-// rz = r.z (tot[0]) and the sum of z over the unknowns (tot[1]) into the
-// Scalars: beta = rz / rz_old (0 on the first iteration or after a restart)
-// and the mean of z for its projection.
-__device__ __forceinline__ void set_rz(Scalars *sc, const double (&tot)[2], int first) {
-  const double old = sc->rz;
-  sc->rz_old = old;
-  sc->rz = tot[0];
-  const double beta = (first || sc->restart || old == 0.0) ? 0.0 : tot[0] / old;
-  sc->restart = 0;
-  sc->beta = beta;
-  sc->beta_f = (float)beta;
-  sc->zsum = tot[1];
-  sc->zmean = tot[1] * sc->inv_ndof;
-  sc->zmean_f = (float)sc->zmean;
-}
-
 template <typename T>
 __global__ void __launch_bounds__(NT)
 k_dot_rz(int nb, const T *__restrict__ r, const T *__restrict__ z,
@@ -344,26 +215,7 @@ k_dot_rz(int nb, const T *__restrict__ r, const T *__restrict__ z,
   }
   const Acc<T> v[2] = {rz, zsum};
   double tot[2];
-  if (grid_sum_acc<T, 2>(v, partials, &sc->ticket[2], tot)) set_rz(sc, tot, first);
-}
-
-// The same scalars from the partial pairs the level-0 post-smoother wrote
-// (k_jacobi7 with RZ): grid-stride sums, then the ticketed block tree.
-template <bool PAIRS>
-__global__ void __launch_bounds__(NT)
-k_finish_rz(const double *__restrict__ partials, int n, double *scratch, Scalars *sc,
-            int first, size_t pstride) {
-  pdl_entry();
-  partials += (size_t)blockIdx.y * pstride;
-  scratch += (size_t)blockIdx.y * pstride;
-  sc += blockIdx.y;
-  double v[2] = {0.0, 0.0};
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    v[0] += pair_at<PAIRS>(partials, 2 * (size_t)i);
-    v[1] += pair_at<PAIRS>(partials, 2 * (size_t)i + 1);
-  }
-  double tot[2];
-  if (grid_sum<2>(v, scratch, &sc->ticket[2], tot)) set_rz(sc, tot, first);
+  if (grid_sum_acc<T, 2>(v, partials, &sc->ticket[2], tot, blockIdx.x, gridDim.x)) set_rz(sc, tot, first);
 }
 
 // Per-component sums of v over the unknowns (several components), exact and
@@ -535,7 +387,7 @@ k_dot(int nb, const T *__restrict__ x, const T *__restrict__ y,
   }
   const Acc<T> v[1] = {acc};
   double tot[1];
-  if (grid_sum_acc<T, 1>(v, partials, &sc->ticket[3], tot)) sc->aux[slot] = tot[0];
+  if (grid_sum_acc<T, 1>(v, partials, &sc->ticket[3], tot, blockIdx.x, gridDim.x)) sc->aux[slot] = tot[0];
 }
 
 // ------------------------------------------------------------ Eq. 3 RHS
@@ -769,7 +621,7 @@ k_energy(const unsigned char *__restrict__ mask, const double *__restrict__ a,
     for (int d = 0; d < 3; ++d) Ev[d * nv + v] = E[d];
   }
   double vals[2] = {sum, cnt}, tot[2];
-  if (grid_sum<2>(vals, partials, &sc->ticket[7], tot)) {
+  if (grid_sum<2>(vals, partials, &sc->ticket[7], tot, blockIdx.x, gridDim.x)) {
     sc->aux[6] = tot[0];
     sc->aux[7] = tot[1];
   }
@@ -934,7 +786,7 @@ k_power27_f32(Grid g, const float *__restrict__ st, const float *__restrict__ di
     two_sum_add(hi[1], lo[1], vs * vs * st[13 * S + s], 0.f);
   }
   double tot[2];
-  if (grid_sum_f32<2>(hi, lo, partials, &sc->ticket[4], tot)) {
+  if (grid_sum_f32<2>(hi, lo, partials, &sc->ticket[4], tot, blockIdx.x, gridDim.x)) {
     sc->aux[4] = tot[0];
     sc->aux[5] = tot[1];
   }
@@ -1035,7 +887,7 @@ k_scale_to_f32(int nb, const double *__restrict__ r, double f,
   }
   const Acc<float> t[1] = {acc};
   double tot[1];
-  if (grid_sum_acc<float, 1>(t, partials, &sc->ticket[5], tot)) {
+  if (grid_sum_acc<float, 1>(t, partials, &sc->ticket[5], tot, blockIdx.x, gridDim.x)) {
     sc->rsum = tot[0];
     sc->rmean = tot[0] * sc->inv_ndof;
     sc->rmean_f = (float)sc->rmean;
@@ -1083,35 +935,28 @@ void launch_scaled_copy(int nb, const double *src, double f, double *dst,
                         cudaStream_t st) {
   if (nb) k_scaled_copy<<<nb, NT, 0, st>>>(src, f, dst);
 }
+static_assert(BV / row_n_apply<float>() == 128 && BV / row_n_jacobi<float>() == 128,
+              "four warps per brick");
+void launch_finish_pairs(bool rz, int nb, const double *pairs, Scalars *sc, int first,
+                         size_t pstride, cudaStream_t st, int nk) {
+  if (!nb) return;
+  const dim3 grid(FP_CLUSTER, nk);
+  if (rz) pdl(k_finish_pairs<2>, grid, FP_THREADS, st)(pairs, 4 * nb, sc, first, pstride);
+  else pdl(k_finish_pairs<1>, grid, FP_THREADS, st)(pairs, 4 * nb, sc, first, pstride);
+}
 template <typename T>
 void launch_apply_dot(const Grid &g, const T *gx, const T *diag, const T *p,
-                      T *q, Scalars *sc, double *partials, cudaStream_t st, int nk,
-                      size_t pstride, int order) {
+                      T *q, Scalars *sc, double *partials, size_t pstride, cudaStream_t st,
+                      int nk, int order) {
   if (!g.nb) return;
+  const int units = sizeof(T) == 4 ? g.nb : walk_units(g.nb, row_min_blocks_apply<T>());
   if (order)
-    pdl(k_apply_dot<T, 1>, unit_grid(1, g.nb, nk), BV / row_n_apply<T>(), st)(
-        g, gx, diag, p, q, sc, partials, pstride, nk);
+    pdl(k_apply_dot<T, 1>, unit_grid(1, units, nk), BV / row_n_apply<T>(), st)(
+        g, gx, diag, p, q, sc, partials, pstride, nk, units);
   else
-    pdl(k_apply_dot<T, 0>, unit_grid(0, g.nb, nk), BV / row_n_apply<T>(), st)(
-        g, gx, diag, p, q, sc, partials, pstride, nk);
-}
-void launch_finish_rz(int n, const double *partials, double *scratch, Scalars *sc, int first,
-                      cudaStream_t st, int nk, size_t pstride, bool pairs) {
-  if (n <= 0) return;
-  const int blocks = std::min(152, (n + NT - 1) / NT);
-  if (pairs)
-    pdl(k_finish_rz<true>, dim3(blocks, nk), NT, st)(partials, n, scratch, sc, first, pstride);
-  else
-    pdl(k_finish_rz<false>, dim3(blocks, nk), NT, st)(partials, n, scratch, sc, first, pstride);
-}
-void launch_finish_pq(int n, const double *partials, double *scratch, Scalars *sc,
-                      cudaStream_t st, int nk, size_t pstride, bool pairs) {
-  if (n <= 0) return;
-  const int blocks = std::min(152, (n + NT - 1) / NT);
-  if (pairs)
-    pdl(k_finish_pq<true>, dim3(blocks, nk), NT, st)(partials, n, scratch, sc, pstride);
-  else
-    pdl(k_finish_pq<false>, dim3(blocks, nk), NT, st)(partials, n, scratch, sc, pstride);
+    pdl(k_apply_dot<T, 0>, unit_grid(0, units, nk), BV / row_n_apply<T>(), st)(
+        g, gx, diag, p, q, sc, partials, pstride, nk, units);
+  if (sizeof(T) == 4) launch_finish_pairs(false, g.nb, partials, sc, 0, pstride, st, nk);
 }
 template <typename T>
 void launch_update_xr(int nb, T *x, T *r, const T *p, const T *q, Scalars *sc,
@@ -1242,7 +1087,7 @@ void launch_energy_grads(const Grid &g, const double *gx, const unsigned char *m
 #define INST_K(T)                                                              \
   template void launch_apply_dot<T>(const Grid &, const T *, const T *,        \
                                     const T *, T *, Scalars *, double *,       \
-                                    cudaStream_t, int, size_t, int);           \
+                                    size_t, cudaStream_t, int, int);           \
   template void launch_update_xr<T>(int, T *, T *, const T *, const T *,       \
                                     Scalars *, double *, cudaStream_t, int,    \
                                     size_t);                                   \
@@ -1263,8 +1108,6 @@ void launch_energy_grads(const Grid &g, const double *gx, const unsigned char *m
                               size_t);                                         \
   template void launch_scatter<T>(const Grid &, const T *, const int *,        \
                                   double *, cudaStream_t, int);
-template int apply_dot_partials<double>(int);
-template int apply_dot_partials<float>(int);
 INST_K(double)
 INST_K(float)
 

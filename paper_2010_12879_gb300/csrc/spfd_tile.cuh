@@ -130,14 +130,15 @@ constexpr int row_threads() { return BV / row_n<T>(); }
 template <typename T>
 constexpr int row_min_blocks() { return sizeof(T) == 4 ? 10 : 4; }
 // The weighted-Jacobi sweep asks for 9 resident FP32 blocks (56 registers,
-// no spills): 61.4 against 65.1 us per level-0 launch on the 2 mm body with
-// 10 (48 registers and spills); the residual and the CG operator measured
-// 2-3 % slower with 9 and keep 10.
+// no spills): with r.z 63.7 us per level-0 launch on the 2 mm body, against
+// 71.6 with 10 (48 registers and spills), 66.5 with 8 and 66.6 with 7; in
+// FP64 for 4 (204 us; 5: 248, 3: 216).  The residual measured 2-3 % slower
+// with 9 and keeps 10.
 template <typename T>
 constexpr int row_min_blocks_jacobi() { return sizeof(T) == 4 ? 9 : 4; }
-// The FP64 CG operator (four nodes per thread) asks for 5 resident blocks (96
-// registers): 190 against 195 us per launch with 4 (108 registers); 6 (80
-// registers and spills) gave 193 us.
+// The CG operator: FP64, whose blocks walk the bricks and keep the p.q sums, 5
+// resident blocks (171 us per launch on the 2 mm body; 4: 171, 6: 214 with
+// spills); FP32 10.
 template <typename T>
 constexpr int row_min_blocks_apply() { return sizeof(T) == 4 ? 10 : 5; }
 
@@ -350,66 +351,6 @@ __device__ __forceinline__ T apply27_tile(const T (*tl)[10][10], const T *__rest
 template <typename T>
 __device__ __forceinline__ T tile_at(const T (*tl)[10][10], int ts) {
   return tl[(ts >> 6) + 1][((ts >> 3) & 7) + 1][(ts & 7) + 1];
-}
-
-// Sum of the N values of every lane of the warp, held by every lane: an
-// FP64 sum for double; for float, an error-free (TwoSum) FP32 pair over the
-// thread's values and the warp.  get() rounds it to FP64.
-template <typename T> struct WarpSum;
-// put() stores the sum into one 8-byte partial slot: the FP64 value, or the
-// FP32 pair (hi, lo) as is, for a finishing kernel that widens it (pair_at)
-// so that the FP32 kernel itself issues no FP64 instruction.
-template <> struct WarpSum<double> {
-  double s;
-  __device__ __forceinline__ double get() const { return s; }
-  __device__ __forceinline__ void put(double *slot) const { *slot = s; }
-};
-template <> struct WarpSum<float> {
-  float hi, lo;
-  __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
-  __device__ __forceinline__ void put(double *slot) const {
-    *reinterpret_cast<float2 *>(slot) = make_float2(hi, lo);
-  }
-};
-// The value of partial slot i: an FP64 value, or (PAIRS) an FP32 pair
-// written by WarpSum<float>::put.
-template <bool PAIRS>
-__device__ __forceinline__ double pair_at(const double *p, size_t i) {
-  if constexpr (PAIRS) {
-    const float2 q = reinterpret_cast<const float2 *>(p)[i];
-    return (double)q.x + (double)q.y;
-  } else {
-    return p[i];
-  }
-}
-template <typename T, int N>
-__device__ __forceinline__ WarpSum<T> warp_total(const T (&v)[N]) {
-  if constexpr (sizeof(T) == 4) {
-    float hi = v[0], lo = 0.f;
-#pragma unroll
-    for (int i = 1; i < N; ++i) {
-      const float sh = hi + v[i], bb = sh - hi;
-      lo += (hi - (sh - bb)) + (v[i] - bb);
-      hi = sh;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float oh = __shfl_xor_sync(0xffffffffu, hi, o);
-      const float ol = __shfl_xor_sync(0xffffffffu, lo, o);
-      const float sh = hi + oh, bb = sh - hi;
-      const float e = (hi - (sh - bb)) + (oh - bb);
-      hi = sh;
-      lo = lo + ol + e;
-    }
-    return WarpSum<float>{hi, lo};
-  } else {
-    double a = v[0];
-#pragma unroll
-    for (int i = 1; i < N; ++i) a += v[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    return WarpSum<double>{a};
-  }
 }
 
 // The 27 entries e * S + s of a direction-major array (stencil coefficients
