@@ -77,7 +77,6 @@ void destroy_ctx(spfd_ctx *c) {
   for (cudaEvent_t e : c->evpool) cudaEventDestroy(e);
   if (c->ev0) cudaEventDestroy(c->ev0);
   if (c->ev1) cudaEventDestroy(c->ev1);
-  if (c->evsc) cudaEventDestroy(c->evsc);
   delete c;
 }
 
@@ -636,11 +635,11 @@ struct PcgResult {
 // The level-0 V-cycle's first kernel, when it depends on nothing but r and
 // the scalars update_xr left on the device (weighted Jacobi, one component,
 // a coarser level below): the projected first sweep from the zero guess.
-// The CG loop launches it right after the scalars' copy to the host, so the
-// GPU runs it while the host waits for the copy and takes its decisions,
-// instead of idling through that round trip; the V-cycle then starts with
-// its residual.  It is the same launch as the V-cycle's own, so results are
-// unchanged bit for bit; when the solve stops there, one sweep is spent.
+// The CG loop launches it right after the x / r update, so the GPU runs it
+// while the host waits for |r|^2 and takes its decisions, instead of idling
+// through that round trip; the V-cycle then starts with its residual.  It is
+// the same launch as the V-cycle's own, so results are unchanged bit for bit;
+// when the solve stops there, one sweep is spent.
 template <typename T>
 static bool vcycle_head_ok(const spfd_ctx *c) {
   return c->opts.smoother == SPFD_SMOOTHER_JACOBI && c->ncomp == 1 && c->L.size() > 1;
@@ -655,6 +654,33 @@ static spfd_status vcycle_head(spfd_ctx *c, T *r, int nk) {
               launch_jacobi_first_proj<T>(lv.g, lv.WDINV<T>(), r, lv.X<T>(), c->sc, inv,
                                           c->stream, nk, block_order(c, TF_JFIRST, 0)));
   return launch_check("first sweep");
+}
+
+// Waits until update number c->seq of every right-hand side still running has
+// written its |r|^2 (HostFlag) to host memory.  Polling the pinned words the
+// kernel writes takes a microsecond or two and puts nothing between the
+// kernels on the stream, where a copy and an event cost 10 to 15 us an
+// iteration.  The stream is queried now and then, so that a failed launch
+// ends the wait.
+static spfd_status wait_update(spfd_ctx *c, int na, const std::vector<int> &done) {
+  auto t0 = std::chrono::steady_clock::now();
+  for (int j = 0; j < na; ++j) {
+    if (done[j]) continue;
+    const HostFlag *h = c->hflag + j;
+    for (unsigned spins = 1; __atomic_load_n(&h->seq, __ATOMIC_ACQUIRE) != c->seq; ++spins) {
+      if (spins % 256) continue;
+      const auto t1 = std::chrono::steady_clock::now();
+      if (t1 - t0 < std::chrono::milliseconds(1)) continue;
+      t0 = t1;
+      const cudaError_t e = cudaStreamQuery(c->stream);
+      if (e == cudaErrorNotReady) continue;
+      if (e != cudaSuccess)
+        return fail(SPFD_ECUDA, "reading solver scalars: %s", cudaGetErrorString(e));
+      if (__atomic_load_n(&h->seq, __ATOMIC_ACQUIRE) != c->seq)
+        return fail(SPFD_EINTERNAL, "the x / r update did not report its residual");
+    }
+  }
+  return launch_check("CG update");
 }
 
 // T = double: the operator is the FP64 one and the stopping rule recomputes
@@ -702,6 +728,7 @@ static spfd_status pcg(spfd_ctx *c, T *x, T *r, T *p, T *q, const T *opgx,
   // rounding floor is reached: stop there (not converged).
   std::vector<double> best_true(nk, INFINITY), min_rrel(nk, INFINITY), rel(nk, 0.0);
   std::vector<int> stall(nk, 0), check, broke;
+  double last[2] = {1.0, 10.0};  // the last two relative residuals (used when nk == 1)
   int maxit_all = 0;
   for (int j = 0; j < nk; ++j) maxit_all = std::max(maxit_all, maxitv[j]);
   for (int it = 1; it <= maxit_all && na > 0; ++it) {
@@ -721,27 +748,34 @@ static spfd_status pcg(spfd_ctx *c, T *x, T *r, T *p, T *q, const T *opgx,
     SPFD_LAUNCH(c, "apply_dot", f32, f32 ? 2 : 1, (f32 ? 5 : 6) * w * S, (f32 ? 20 : 15) * S,
                 launch_apply_dot<T>(l0.g, opgx, opdiag, p, q, c->sc, c->partials, c->pstride, st,
                                     na, block_order(c, TF_APPLY, 0)));
+    ++c->seq;
     SPFD_LAUNCH(c, "update_xr", f32, 1, 6 * w * S, 7 * S,
-                launch_update_xr<T>(nb, x, r, p, q, c->sc, c->partials, st, na, c->pstride));
+                launch_update_xr<T>(nb, x, r, p, q, c->sc, c->partials, st, na, c->pstride,
+                                    c->hflag, c->seq));
     TRY(launch_check("CG update"));
-    CU(cudaMemcpyAsync(c->hsc, c->sc, (size_t)na * sizeof(Scalars), cudaMemcpyDeviceToHost,
-                       st));
-    CU(cudaEventRecord(c->evsc, st));
-    if (ahead) TRY(vcycle_head<T>(c, r, na));
-    bool head = ahead;  // false once the host replaces an r (restart)
-    {
-      cudaError_t e = cudaEventSynchronize(c->evsc);
-      if (e == cudaSuccess) e = cudaGetLastError();
-      if (e != cudaSuccess)
-        return fail(SPFD_ECUDA, "reading solver scalars: %s", cudaGetErrorString(e));
+    // A single right-hand side that, going by its last two residuals, cannot
+    // have converged yet gets its whole preconditioning step launched before
+    // the host knows |r|^2 (none of it touches x, and a restart repeats it);
+    // else the first sweep is, if it may (see vcycle_head).
+    const bool spec = nk == 1 && last[0] * std::min(1.0, last[0] / last[1]) > 4.0 * tolv[0];
+    bool head = false;  // false once the host replaces an r (restart)
+    if (spec) {
+      TRY(precondition(0, false));
+    } else if (ahead) {
+      TRY(vcycle_head<T>(c, r, na));
+      head = true;
     }
+    TRY(wait_update(c, na, done));
+    bool prec = spec;  // the preconditioning step is on the stream
     check.clear();
     broke.clear();
     for (int j = 0; j < na; ++j) {
       if (done[j]) continue;
       res[j].iters = it;
       const double tol = tolv[j];
-      const double rrel = std::sqrt(c->hsc[j].rr / bb[j]);
+      const double rrel = std::sqrt(c->hflag[j].rr / bb[j]);
+      last[1] = last[0];
+      last[0] = rrel;
       if (!std::isfinite(rrel) || rrel > 1e8 * std::max(min_rrel[j], tol)) {
         broke.push_back(j);  // breakdown: report the current iterate, not converged
         continue;
@@ -768,6 +802,7 @@ static spfd_status pcg(spfd_ctx *c, T *x, T *r, T *p, T *q, const T *opgx,
                          cudaMemcpyDeviceToDevice, st));
       TRY(project<T>(c, r + (size_t)j * S0, 1, j));
       TRY(batch_flags(c, j, 1, 1, -1, 1));
+      prec = false;
       if (head) {
         // the V-cycle runs the first sweep again: the other right-hand
         // sides' r were projected by the look-ahead sweep, so their means
@@ -782,7 +817,7 @@ static spfd_status pcg(spfd_ctx *c, T *x, T *r, T *p, T *q, const T *opgx,
         done[j] = 2;
       }
     na = active_end();
-    if (na > 0) TRY(precondition(0, head));
+    if (na > 0 && !prec) TRY(precondition(0, head));
   }
   return SPFD_OK;
 }
@@ -1006,6 +1041,8 @@ static spfd_status ensure_batch(spfd_ctx *c, int k) {
   c->sc = sc;
   ++c->gen;  // solve buffers moved: captured graphs must be captured again
   c->hsc = hsc;
+  TRY(halloc(c, &c->hflag, k));
+  memset(c->hflag, 0, (size_t)k * sizeof(HostFlag));
   c->kcap = k;
   return SPFD_OK;
 }

@@ -442,9 +442,10 @@ spfd_status build_impl(spfd_ctx *c, const double *sigma) {
   CU(cudaMemsetAsync(c->sc, 0, sizeof(Scalars), st));
   TRY(halloc(c, &c->hsc, 1));
   memset(c->hsc, 0, sizeof(Scalars));
+  TRY(halloc(c, &c->hflag, 1));
+  memset(c->hflag, 0, sizeof(HostFlag));
   CU(cudaEventCreate(&c->ev0));
   CU(cudaEventCreate(&c->ev1));
-  CU(cudaEventCreateWithFlags(&c->evsc, cudaEventDisableTiming));
   CU(cudaEventRecord(c->ev0, st));
   const int64_t launches0 = c->launch_count;
 

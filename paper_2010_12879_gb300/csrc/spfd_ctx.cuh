@@ -148,6 +148,8 @@ struct spfd_ctx {
   float *dk32 = nullptr, *rk32 = nullptr, *pk32 = nullptr, *qk32 = nullptr;
   spfd::Scalars *sc = nullptr;    // device scalars, one per right-hand side
   spfd::Scalars *hsc = nullptr;   // pinned host mirror
+  spfd::HostFlag *hflag = nullptr;  // pinned, one per right-hand side (CG loop)
+  unsigned seq = 0;               // number of the last x / r update
   double *partials = nullptr;     // reduction scratch, pstride per right-hand side
   size_t pstride = 0;
   // right-hand sides the per-RHS buffers hold (level vectors, Krylov
@@ -186,7 +188,6 @@ struct spfd_ctx {
   const signed char *ord = nullptr;
   std::vector<spfd::TuneRecord> tune_log;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-  cudaEvent_t evsc = nullptr;  // the CG scalars' copy to the host
   spfd_info info{};
   // launch accounting and profiling
   int64_t launch_count = 0;

@@ -677,9 +677,12 @@ k_coarse_solve(int m, size_t S, const int *__restrict__ idx, const double *__res
 // 8.9 / 10.9 against 7.3 / 8.1 / 10.2; 4068 bricks FP64 66.9 / 71.4 against
 // 88.6 / 100, FP32 35.1 / 38.9 against 37.3 / 43.2 (there a brick's four
 // halos cost more than they save, and FP64 compaction works on fewer slots).
+// Captured solves run beside other bodies' kernels, where throughput counts
+// more than latency: 12 uneven bodies as one graph took 21.3 ms with no
+// quarter bricks, 21.2 up to 100 bricks, 21.4 up to 300, 21.7 up to 1000.
 template <typename T>
-constexpr bool slab_level(int nb, int nk, bool resid) {
-  return (long long)nb * nk <= (sizeof(T) == 4 || resid ? 1000 : 512);
+bool slab_level(int nb, int nk, bool resid) {
+  return (long long)nb * nk <= (!pdl_allowed ? 100 : sizeof(T) == 4 || resid ? 1000 : 512);
 }
 template <typename T, typename C>
 void launch_residual7(const Grid &g, const C *gx, const T *diag, const T *x,

@@ -364,6 +364,14 @@ struct Scalars {
   int restart;      // batched solves: the next beta of this right-hand side is 0
 };
 
+// What the host reads of a CG iteration, in pinned host memory that the last
+// block of the x / r update writes: |r|^2, then the number of that update.
+struct HostFlag {
+  double rr;
+  unsigned seq;
+  unsigned pad;
+};
+
 enum : int {
   DEV_BAD_SIGMA = 1,     // NaN / negative / infinite conductivity
   DEV_BAD_A = 2,         // non-finite edge potential on a conducting edge
@@ -557,10 +565,12 @@ void launch_apply_dot(const Grid &g, const T *gx, const T *diag, const T *p,
 void launch_finish_pairs(bool rz, int nb, const double *pairs, Scalars *sc, int first,
                          size_t pstride, cudaStream_t st, int nk);
 // x += alpha p, r -= alpha q, r.r, sum r; right-hand sides whose Scalars are
-// frozen are left as they are.
+// frozen are left as they are.  hf (one per right-hand side, may be null)
+// receives r.r and seq.
 template <typename T>
 void launch_update_xr(int nb, T *x, T *r, const T *p, const T *q, Scalars *sc,
-                      double *partials, cudaStream_t st, int nk = 1, size_t pstride = 0);
+                      double *partials, cudaStream_t st, int nk = 1, size_t pstride = 0,
+                      HostFlag *hf = nullptr, unsigned seq = 0);
 // r.z and beta (0 when first, or when the right-hand side's restart flag is
 // set; the flag is cleared).
 template <typename T>

@@ -145,7 +145,7 @@ template <typename T>
 __global__ void __launch_bounds__(NT)
 k_update_xr(int nb, T *__restrict__ x, T *__restrict__ r,
             const T *__restrict__ p, const T *__restrict__ q, Scalars *sc,
-            double *partials, size_t pstride) {
+            double *partials, size_t pstride, HostFlag *hf, unsigned seq) {
   pdl_entry();
   constexpr int N = V16<T>::N;
   sc += blockIdx.y;
@@ -177,6 +177,12 @@ k_update_xr(int nb, T *__restrict__ x, T *__restrict__ r,
   const Acc<T> v[2] = {rr, rs_sum};
   double tot[2];
   if (grid_sum_acc<T, 2>(v, partials, &sc->ticket[1], tot, blockIdx.x, gridDim.x)) {
+    if (hf) {  // r.r before its number: the host reads them in the other order
+      volatile HostFlag *h = hf + blockIdx.y;
+      h->rr = tot[0];
+      __threadfence_system();
+      h->seq = seq;
+    }
     sc->rr = tot[0];
     sc->rsum = tot[1];
     sc->rmean = tot[1] * sc->inv_ndof;
@@ -960,10 +966,11 @@ void launch_apply_dot(const Grid &g, const T *gx, const T *diag, const T *p,
 }
 template <typename T>
 void launch_update_xr(int nb, T *x, T *r, const T *p, const T *q, Scalars *sc,
-                      double *partials, cudaStream_t st, int nk, size_t pstride) {
+                      double *partials, cudaStream_t st, int nk, size_t pstride, HostFlag *hf,
+                      unsigned seq) {
   if (nb)
-    pdl(k_update_xr<T>, dim3(std::min(nb, RED_GRID), nk), NT, st)(nb, x, r, p, q, sc,
-                                                                    partials, pstride);
+    pdl(k_update_xr<T>, dim3(std::min(nb, RED_GRID), nk), NT, st)(nb, x, r, p, q, sc, partials,
+                                                                  pstride, hf, seq);
 }
 template <typename T>
 void launch_dot_rz(int nb, const T *r, const T *z, const int *comp,
@@ -1090,7 +1097,7 @@ void launch_energy_grads(const Grid &g, const double *gx, const unsigned char *m
                                     size_t, cudaStream_t, int, int);           \
   template void launch_update_xr<T>(int, T *, T *, const T *, const T *,       \
                                     Scalars *, double *, cudaStream_t, int,    \
-                                    size_t);                                   \
+                                    size_t, HostFlag *, unsigned);             \
   template void launch_dot_rz<T>(int, const T *, const T *, const int *,       \
                                  Scalars *, double *, int, cudaStream_t, int,  \
                                  size_t);                                      \
