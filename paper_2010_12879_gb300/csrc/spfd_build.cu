@@ -374,10 +374,12 @@ static spfd_status setup_coarsest(spfd_ctx *c, PhaseClock &clk, double **spare) 
   TRY(dalloc(c, &b1, (size_t)m * m));
   double *inv = nullptr;
   unsigned *bar = nullptr;
+  double *dinv = nullptr;
+  TRY(dalloc(c, &dinv, 512));
   TRY(dalloc(c, &bar, 2));
   CU(cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), c->stream));
   SPFD_LAUNCH(c, "setup_coarsest", false, dense_inverse_launches(m), 0, 2.0 * m * m * m,
-              inv = launch_dense_inverse(b0, b1, m, &c->sc->status, bar, c->stream));
+              inv = launch_dense_inverse(b0, b1, m, dinv, &c->sc->status, bar, c->stream));
   TRY(launch_check("coarsest inverse"));
   // a non-positive pivot raises DEV_BAD_PIVOT, read at the end of the build
   c->Binv = inv;

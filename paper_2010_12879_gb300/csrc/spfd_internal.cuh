@@ -473,9 +473,9 @@ void launch_coarse_dense(const Grid &g, const double *op, bool k27, size_t S, co
                          const double *mu, double shift, double *A, cudaStream_t st);
 // Inverse of the SPD matrix in buf0 (m x m, row-major) by blocked
 // Gauss-Jordan sweeps; returns buf0 or buf1, whichever holds the result.
-// bar: two zeroed unsigned ints.
-double *launch_dense_inverse(double *buf0, double *buf1, int m, int *status, unsigned *bar,
-                             cudaStream_t st);
+// dinv: 512 doubles of scratch; bar: two zeroed unsigned ints.
+double *launch_dense_inverse(double *buf0, double *buf1, int m, double *dinv, int *status,
+                             unsigned *bar, cudaStream_t st);
 int dense_inverse_launches(int m);
 
 // V-cycle pieces (spfd_cycle.cu); T = vector type, C = 7-point coefficient type.

@@ -550,132 +550,98 @@ void launch_coarse_dense(const Grid &g, const double *op, bool k27, size_t S, co
 // After every pivot set has been swept once, B = A^-1.  D is inverted by
 // scalar Gauss-Jordan in shared memory: its pivots are Schur complements of
 // the SPD matrix, hence positive; a non-positive one raises DEV_BAD_PIVOT.
-// Every block inverts D itself, forms W = D^-1 M[K, its columns] and
-// updates its GJ_T x GJ_T tile; sweeps run one launch each (k_gj_block) or
-// all in one cooperative launch with a grid barrier between them (k_gj_all).
-// (Forming D^-1 and W once per column tile in a first phase of each sweep
-// halves the FP64 work, but its second grid barrier per sweep made the
-// inversion of the 2 mm body's 481 x 481 coarsest matrix slower: the sweeps
-// are bound by latency, not by the FP64 pipe.)
+// Sweeps run in one cooperative launch (k_gj_strips) or, for large m, one
+// launch each (k_gj_block, where every block inverts D itself); the order of
+// every sum is the same in both.
 constexpr int GJ_B = 16;   // pivots per sweep
 constexpr int GJ_T = 32;   // tile edge
 constexpr int GJ_NT = 256; // threads per block (GJ_B * GJ_B)
 
-struct GjShared {
+// D <- D^-1 in shared memory, one pivot per step, ping-pong between D[0] and
+// D[1] (entry D[0] and pinv[0], the reciprocal of its first pivot, are in
+// place; a barrier comes first): the thread that forms the next pivot also
+// writes its reciprocal, so a step needs a single barrier.  The inverse ends
+// in D[GJ_B & 1] = D[0].
+struct GjPivots {
   double D[2][GJ_B][GJ_B + 1];
-  double W[GJ_B][GJ_T];
-  double U[GJ_T][GJ_B + 1];
-  double C[GJ_B][GJ_T];
   double pinv[2];
 };
-
-// COH: read through L2 only (ld.global.cg), as the single-launch form must:
-// what it reads was written by other blocks in the same launch, and a line
-// cached in this SM's L1 by an earlier sweep would be stale.
-template <bool COH>
-__device__ __forceinline__ double gj_ld(const double *p) {
-  if constexpr (COH) return __ldcg(p);
-  else return *p;
-}
-
-// D = M[K,K] (identity-padded to GJ_B) into sh.D[0] and its first pivot's
-// reciprocal, and C = M[K, column tile j0] into sh.C.  A barrier follows.
-template <bool COH>
-__device__ __forceinline__ void gj_load_pivot_rows(GjShared &sh, const double *__restrict__ A,
-                                                   int m, int k0, int r, int j0, int *status) {
-  const int t = threadIdx.x;
-  const int a = t / GJ_B, b = t % GJ_B;
-  const double d0 =
-      (a < r && b < r) ? gj_ld<COH>(&A[(size_t)(k0 + a) * m + k0 + b]) : (a == b ? 1.0 : 0.0);
-  sh.D[0][a][b] = d0;
-  if (t == 0) {
+__device__ __forceinline__ void gj_first_pivot(GjPivots &s, double d0, int *status) {
+  s.D[0][threadIdx.x / GJ_B][threadIdx.x % GJ_B] = d0;
+  if (threadIdx.x == 0) {
     if (!(d0 > 0.0)) atomicOr(status, DEV_BAD_PIVOT);
-    sh.pinv[0] = d0 > 0.0 ? 1.0 / d0 : 0.0;
-  }
-  for (int q = t; q < GJ_T * GJ_B; q += GJ_NT) {
-    const int l2 = q / GJ_T, jj = q % GJ_T;
-    sh.C[l2][jj] =
-        (l2 < r && j0 + jj < m) ? gj_ld<COH>(&A[(size_t)(k0 + l2) * m + j0 + jj]) : 0.0;
+    s.pinv[0] = d0 > 0.0 ? 1.0 / d0 : 0.0;
   }
 }
-
-// U = M[tile rows i0, K] into sh.U.  A barrier follows.
-template <bool COH>
-__device__ __forceinline__ void gj_load_pivot_cols(GjShared &sh, const double *__restrict__ A,
-                                                   int m, int k0, int r, int i0) {
-  for (int q = threadIdx.x; q < GJ_T * GJ_B; q += GJ_NT) {
-    const int ii = q / GJ_B, l = q % GJ_B;
-    sh.U[ii][l] = (l < r && i0 + ii < m) ? gj_ld<COH>(&A[(size_t)(i0 + ii) * m + k0 + l]) : 0.0;
-  }
-}
-
-// D <- D^-1 in shared memory (after a barrier), one pivot per step,
-// ping-pong between D[0] and D[1]: the thread that forms the next pivot also
-// writes its reciprocal, so a step needs a single barrier.  The inverse ends
-// in D[GJ_B & 1] = D[0]; W = D^-1 C then follows (each thread forms the
-// entries (l, jj) and (l + 8, jj), its two sums interleaved, each in its own
-// fixed order), and a barrier.
-__device__ __forceinline__ void gj_invert_pivots(GjShared &sh, int *status) {
-  auto &D = sh.D;
-  auto &pinv = sh.pinv;
-  const int t = threadIdx.x;
-  const int a = t / GJ_B, b = t % GJ_B;
+__device__ __forceinline__ void gj_invert_pivots(GjPivots &s, int *status) {
+  const int a = threadIdx.x / GJ_B, b = threadIdx.x % GJ_B;
+  __syncthreads();
   for (int p = 0; p < GJ_B; ++p) {
-    const double(*Dc)[GJ_B + 1] = D[p & 1];
-    const double iv = pinv[p & 1];
+    const double(*Dc)[GJ_B + 1] = s.D[p & 1];
+    const double iv = s.pinv[p & 1];
     double v;
     if (a == p && b == p) v = iv;
     else if (a == p) v = Dc[p][b] * iv;
     else if (b == p) v = -Dc[a][p] * iv;
     else v = Dc[a][b] - Dc[a][p] * Dc[p][b] * iv;
-    D[(p + 1) & 1][a][b] = v;
+    s.D[(p + 1) & 1][a][b] = v;
     if (a == p + 1 && b == p + 1) {
       if (!(v > 0.0)) atomicOr(status, DEV_BAD_PIVOT);
-      pinv[(p + 1) & 1] = v > 0.0 ? 1.0 / v : 0.0;
+      s.pinv[(p + 1) & 1] = v > 0.0 ? 1.0 / v : 0.0;
     }
     __syncthreads();
   }
-  const double(*Dinv)[GJ_B + 1] = D[GJ_B & 1];
-  static_assert(GJ_B * GJ_T == 2 * GJ_NT && GJ_T * GJ_T == 4 * GJ_NT, "tile shape");
+}
+
+// One sweep per launch, a GJ_T x GJ_T tile per block: D^-1, W = D^-1 M[K, the
+// tile's columns], then rows ii0 + 8k (k = 0..3) of column jj, four
+// independent chains per thread, each subtracting its terms in order l =
+// 0..15.
+__global__ void __launch_bounds__(GJ_NT)
+k_gj_block(const double *__restrict__ A, double *__restrict__ B, int m, int k0, int r,
+           int *status) {
+  __shared__ GjPivots pv;
+  __shared__ double W[GJ_B][GJ_T], U[GJ_T][GJ_B + 1], C[GJ_B][GJ_T];
+  const int i0 = blockIdx.y * GJ_T, j0 = blockIdx.x * GJ_T, t = threadIdx.x;
   {
-    const int l = t / GJ_T, jj = t % GJ_T;
+    const int a = t / GJ_B, b = t % GJ_B;
+    gj_first_pivot(pv, (a < r && b < r) ? A[(size_t)(k0 + a) * m + k0 + b] : (a == b ? 1.0 : 0.0),
+                   status);
+  }
+  for (int q = t; q < GJ_T * GJ_B; q += GJ_NT) {
+    const int l2 = q / GJ_T, jj = q % GJ_T, ii = q / GJ_B, l = q % GJ_B;
+    C[l2][jj] = (l2 < r && j0 + jj < m) ? A[(size_t)(k0 + l2) * m + j0 + jj] : 0.0;
+    U[ii][l] = (l < r && i0 + ii < m) ? A[(size_t)(i0 + ii) * m + k0 + l] : 0.0;
+  }
+  gj_invert_pivots(pv, status);
+  const double(*Dinv)[GJ_B + 1] = pv.D[GJ_B & 1];
+  static_assert(GJ_B * GJ_T == 2 * GJ_NT && GJ_T * GJ_T == 4 * GJ_NT, "tile shape");
+  constexpr int RS = GJ_NT / GJ_T;  // row stride between a thread's entries
+  const int ii0 = t / GJ_T, jj = t % GJ_T, j = j0 + jj;
+  {
     double w0 = 0.0, w1 = 0.0;
 #pragma unroll
     for (int l2 = 0; l2 < GJ_B; ++l2) {
-      const double c = sh.C[l2][jj];
-      w0 += Dinv[l][l2] * c;
-      w1 += Dinv[l + GJ_NT / GJ_T][l2] * c;
+      const double c = C[l2][jj];
+      w0 += Dinv[ii0][l2] * c;
+      w1 += Dinv[ii0 + RS][l2] * c;
     }
-    sh.W[l][jj] = w0;
-    sh.W[l + GJ_NT / GJ_T][jj] = w1;
+    W[ii0][jj] = w0;
+    W[ii0 + RS][jj] = w1;
   }
   __syncthreads();
-}
-
-// The tile (i0, j0) of B from M (A), with D^-1 in sh.D[0], W for the
-// tile's columns in sh.W and U in sh.U: each thread updates rows ii0 + 8k
-// (k = 0..3) of column jj, four independent chains, each subtracting its
-// terms in order l = 0..15.
-template <bool COH>
-__device__ __forceinline__ void gj_update_tile(const GjShared &sh, const double *__restrict__ A,
-                                               double *__restrict__ B, int m, int k0, int r,
-                                               int i0, int j0) {
-  const double(*Dinv)[GJ_B + 1] = sh.D[GJ_B & 1];
-  constexpr int RS = GJ_NT / GJ_T;  // row stride between a thread's entries
-  const int t = threadIdx.x;
-  const int ii0 = t / GJ_T, jj = t % GJ_T, j = j0 + jj;
   const bool kj = j >= k0 && j < k0 + r;
   double v[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int i = i0 + ii0 + RS * k;
-    v[k] = (!kj && i < m && j < m) ? gj_ld<COH>(&A[(size_t)i * m + j]) : 0.0;
+    v[k] = (!kj && i < m && j < m) ? A[(size_t)i * m + j] : 0.0;
   }
 #pragma unroll
   for (int l = 0; l < GJ_B; ++l) {
-    const double mc = kj ? Dinv[l][j - k0] : sh.W[l][jj];
+    const double mc = kj ? Dinv[l][j - k0] : W[l][jj];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] -= sh.U[ii0 + RS * k][l] * mc;
+    for (int k = 0; k < 4; ++k) v[k] -= U[ii0 + RS * k][l] * mc;
   }
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
@@ -683,77 +649,173 @@ __device__ __forceinline__ void gj_update_tile(const GjShared &sh, const double 
     if (i >= m || j >= m) continue;
     const bool ki = i >= k0 && i < k0 + r;
     double out = v[k];
-    if (ki) out = kj ? Dinv[i - k0][j - k0] : sh.W[i - k0][jj];
+    if (ki) out = kj ? Dinv[i - k0][j - k0] : W[i - k0][jj];
     B[(size_t)i * m + j] = out;
   }
 }
 
-// One sweep per launch: every block forms D^-1 and its W itself.
-__global__ void __launch_bounds__(GJ_NT)
-k_gj_block(const double *__restrict__ A, double *__restrict__ B, int m, int k0, int r,
-           int *status) {
-  __shared__ GjShared sh;
-  const int i0 = blockIdx.y * GJ_T, j0 = blockIdx.x * GJ_T;
-  gj_load_pivot_rows<false>(sh, A, m, k0, r, j0, status);
-  gj_load_pivot_cols<false>(sh, A, m, k0, r, i0);
-  __syncthreads();
-  gj_invert_pivots(sh, status);
-  gj_update_tile<false>(sh, A, B, m, k0, r, i0, j0);
+// Every sweep in one cooperative launch, with a grid barrier between sweeps.
+// Block s updates the four columns 4s .. 4s + 3 over all rows, and one block
+// more forms the next sweep's D (its 16 x 16 entries updated as any other)
+// and inverts it meanwhile, so that the inversion's 16 dependent steps are
+// off the update's path and done once.  With a 32 x 32 tile per block, each
+// inverting D itself (256 blocks for the 481 unknowns of the 2 mm body's
+// coarsest level, two on most SMs), a sweep took 25 to 28 us, of which 15 us
+// FP64 pipe; here the pipe needs 8 us an SM: M[., K] goes to shared memory
+// once per block, W is 64 sums, and a thread carries eight independent chains.
+// dinv: two 16 x 16 buffers; bar: barrier counter and generation, zero at
+// launch.  Reads of the matrix go through L2 (ld.global.cg): other blocks
+// wrote it in the previous sweep.
+constexpr int GS_W = 4;                  // columns per block
+constexpr int GS_R = GJ_NT / GS_W;       // rows per pass of the block
+constexpr int GS_K = 8;                  // rows per thread and chunk
+constexpr int GS_MAX = 1024;             // largest m (shared memory: 136 bytes per row)
+// rows up to the last chunk's end: a thread reads (and discards) U past row m
+constexpr size_t gs_smem(int m) {
+  return (size_t)((m + GS_R * GS_K - 1) / (GS_R * GS_K)) * (GS_R * GS_K) * (GJ_B + 1) *
+         sizeof(double);
 }
 
-// Every sweep in one cooperative launch: the same tiles and arithmetic as
-// the per-sweep launches, with a grid barrier between sweeps (sweep k reads
-// what sweep k-1 wrote).  bar[0..1]: barrier counter and generation, zero
-// at launch.
-__global__ void __launch_bounds__(GJ_NT)
-k_gj_all(double *buf0, double *buf1, int m, int *status, unsigned *bar) {
-  __shared__ GjShared sh;
-  const unsigned nblocks = gridDim.x * gridDim.y;
-  const int i0 = blockIdx.y * GJ_T, j0 = blockIdx.x * GJ_T;
-  double *a = buf0, *b = buf1;
-  for (int k0 = 0; k0 < m; k0 += GJ_B) {
-    const int r = m - k0 < GJ_B ? m - k0 : GJ_B;
-    gj_load_pivot_rows<true>(sh, a, m, k0, r, j0, status);
-    gj_load_pivot_cols<true>(sh, a, m, k0, r, i0);
-    __syncthreads();
-    gj_invert_pivots(sh, status);
-    gj_update_tile<true>(sh, a, b, m, k0, r, i0, j0);
-    grid_barrier(&bar[0], &bar[1], nblocks, status);
-    double *tmp = a; a = b; b = tmp;
+// Rows row0 + GS_R k (k < NK) of column j: v -= U W, in order l = 0..15.
+template <int NK>
+__device__ __forceinline__ void gs_update(const double *__restrict__ U, const double *wc,
+                                          int wstride, int row0, double (&v)[GS_K]) {
+#pragma unroll
+  for (int l = 0; l < GJ_B; ++l) {
+    const double mc = wc[l * wstride];
+#pragma unroll
+    for (int k = 0; k < NK; ++k) v[k] -= U[(row0 + GS_R * k) * (GJ_B + 1) + l] * mc;
   }
 }
 
-// Kernel launches of launch_dense_inverse for an m x m matrix: one when its
-// tile grid fits on the device at once (a cooperative launch), else one per
-// pivot set.
-int dense_inverse_launches(int m) {
-  const int nt = (m + GJ_T - 1) / GJ_T;
+__global__ void __launch_bounds__(GJ_NT)
+k_gj_strips(double *buf0, double *buf1, int m, double *dinv, int *status, unsigned *bar) {
+  extern __shared__ double U[];  // [m rounded up][GJ_B + 1]
+  __shared__ GjPivots pv;
+  __shared__ double Ds[GJ_B][GJ_B + 1], W[GJ_B][GS_W], C[GJ_B][GS_W], Cn[GJ_B][GJ_B + 1];
+  const int t = threadIdx.x, a = t / GJ_B, b = t % GJ_B;
+  const bool pivot = blockIdx.x == gridDim.x - 1;
+  const int j0 = blockIdx.x * GS_W, jj = t % GS_W, j = j0 + jj, rg = t / GS_W;
+  double *A = buf0, *B = buf1;
+  if (pivot) {  // the first sweep's D^-1
+    const int r = min(GJ_B, m);
+    gj_first_pivot(pv, (a < r && b < r) ? __ldcg(&A[(size_t)a * m + b]) : (a == b ? 1.0 : 0.0),
+                   status);
+    gj_invert_pivots(pv, status);
+    dinv[t] = pv.D[GJ_B & 1][a][b];
+  }
+  grid_barrier(&bar[0], &bar[1], gridDim.x, status);
+  for (int k0 = 0, sw = 0; k0 < m; k0 += GJ_B, ++sw) {
+    const int r = min(GJ_B, m - k0);
+    const double *Dg = dinv + (sw & 1) * GJ_NT;
+    Ds[a][b] = __ldcg(&Dg[t]);
+    if (pivot) {
+      const int k1 = k0 + GJ_B, r1 = min(GJ_B, m - k1);
+      if (r1 > 0) {  // the last sweep has no successor (and r == GJ_B here)
+        double(*Un)[GJ_B + 1] = reinterpret_cast<double(*)[GJ_B + 1]>(U);
+        Cn[a][b] = b < r1 ? __ldcg(&A[(size_t)(k0 + a) * m + k1 + b]) : 0.0;
+        Un[a][b] = a < r1 ? __ldcg(&A[(size_t)(k1 + a) * m + k0 + b]) : 0.0;
+        double v = (a < r1 && b < r1) ? __ldcg(&A[(size_t)(k1 + a) * m + k1 + b]) : 0.0;
+        __syncthreads();
+        double w = 0.0;
+#pragma unroll
+        for (int l2 = 0; l2 < GJ_B; ++l2) w += Ds[a][l2] * Cn[l2][b];
+        __syncthreads();
+        Cn[a][b] = w;
+        __syncthreads();
+#pragma unroll
+        for (int l = 0; l < GJ_B; ++l) v -= Un[a][l] * Cn[l][b];
+        gj_first_pivot(pv, (a < r1 && b < r1) ? v : (a == b ? 1.0 : 0.0), status);
+        gj_invert_pivots(pv, status);
+        dinv[((sw + 1) & 1) * GJ_NT + t] = pv.D[GJ_B & 1][a][b];
+      }
+    } else {
+      if (t < GJ_B * GS_W) {
+        const int l2 = t / GS_W;
+        C[l2][jj] = (l2 < r && j < m) ? __ldcg(&A[(size_t)(k0 + l2) * m + j]) : 0.0;
+      }
+#pragma unroll 8
+      for (int q = t; q < m * GJ_B; q += GJ_NT) {
+        const int row = q / GJ_B, l = q % GJ_B;
+        U[row * (GJ_B + 1) + l] = l < r ? __ldcg(&A[(size_t)row * m + k0 + l]) : 0.0;
+      }
+      const bool kj = j >= k0 && j < k0 + r;
+      double v[GS_K];
+      auto load = [&](int base) {
+#pragma unroll
+        for (int k = 0; k < GS_K; ++k) {
+          const int i = base + rg + GS_R * k;
+          v[k] = (!kj && i < m && j < m) ? __ldcg(&A[(size_t)i * m + j]) : 0.0;
+        }
+      };
+      load(0);
+      __syncthreads();
+      if (t < GJ_B * GS_W) {
+        const int l = t / GS_W;
+        double w = 0.0;
+#pragma unroll
+        for (int l2 = 0; l2 < GJ_B; ++l2) w += Ds[l][l2] * C[l2][jj];
+        W[l][jj] = w;
+      }
+      __syncthreads();
+      const double *wc = kj ? &Ds[0][j - k0] : &W[0][jj];
+      const int ws = kj ? GJ_B + 1 : GS_W;
+      for (int base = 0; base < m; base += GS_R * GS_K) {
+        if (base) load(base);
+        // rows this warp has left, uniform: its first row and every GS_R-th
+        const int left = m - base - (t & ~31) / GS_W;
+        const int nk = left <= 0 ? 0 : (left + GS_R - 1) / GS_R;
+        if (nk >= GS_K) gs_update<GS_K>(U, wc, ws, base + rg, v);
+        else if (nk == GS_K - 1) gs_update<GS_K - 1>(U, wc, ws, base + rg, v);
+        else if (nk > GS_K / 2) gs_update<GS_K - 2>(U, wc, ws, base + rg, v);
+        else if (nk > 0) gs_update<GS_K / 2>(U, wc, ws, base + rg, v);
+#pragma unroll
+        for (int k = 0; k < GS_K; ++k) {
+          const int i = base + rg + GS_R * k;
+          if (i >= m || j >= m) continue;
+          const bool ki = i >= k0 && i < k0 + r;
+          B[(size_t)i * m + j] = ki ? wc[(i - k0) * ws] : v[k];
+        }
+      }
+    }
+    grid_barrier(&bar[0], &bar[1], gridDim.x, status);
+    double *tmp = A; A = B; B = tmp;
+  }
+}
+
+// Whether the m x m inverse runs as one cooperative launch: its blocks have
+// to be resident all at once.
+static bool gj_one_launch(int m) {
   int dev = 0, nsm = 0, per_sm = 0, coop = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gj_all, GJ_NT, 0) !=
-          cudaSuccess) {
-    cudaGetLastError();
-    return (m + GJ_B - 1) / GJ_B;
-  }
-  return (coop && (long long)nt * nt <= (long long)per_sm * nsm) ? 1 : (m + GJ_B - 1) / GJ_B;
+  if (m <= GS_MAX && cudaGetDevice(&dev) == cudaSuccess &&
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
+      cudaFuncSetAttribute(k_gj_strips, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)gs_smem(GS_MAX)) == cudaSuccess &&
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gj_strips, GJ_NT, gs_smem(m)) ==
+          cudaSuccess)
+    return (m + GS_W - 1) / GS_W + 1 <= per_sm * nsm;
+  cudaGetLastError();
+  return false;
 }
+
+// Kernel launches of launch_dense_inverse for an m x m matrix.
+int dense_inverse_launches(int m) { return gj_one_launch(m) ? 1 : (m + GJ_B - 1) / GJ_B; }
 
 // Inverts the SPD matrix in buf0 (m x m); returns the buffer holding A^-1
-// (buf0 or buf1, which serve as ping-pong buffers).  bar: two zeroed
-// unsigned ints of device scratch for the cooperative form.
-double *launch_dense_inverse(double *buf0, double *buf1, int m, int *status, unsigned *bar,
-                             cudaStream_t st) {
+// (buf0 or buf1, which serve as ping-pong buffers).  dinv: 512 doubles and
+// bar: two zeroed unsigned ints of device scratch for the cooperative form.
+double *launch_dense_inverse(double *buf0, double *buf1, int m, double *dinv, int *status,
+                             unsigned *bar, cudaStream_t st) {
   double *a = buf0, *b = buf1;
-  const int nt = (m + GJ_T - 1) / GJ_T;
-  if (dense_inverse_launches(m) == 1) {
-    void *args[] = {&buf0, &buf1, &m, &status, &bar};
-    if (cudaLaunchCooperativeKernel((const void *)k_gj_all, dim3(nt, nt), dim3(GJ_NT), args, 0,
-                                    st) == cudaSuccess)
+  if (gj_one_launch(m)) {
+    void *args[] = {&buf0, &buf1, &m, &dinv, &status, &bar};
+    if (cudaLaunchCooperativeKernel((const void *)k_gj_strips, dim3((m + GS_W - 1) / GS_W + 1),
+                                    dim3(GJ_NT), args, gs_smem(m), st) == cudaSuccess)
       return ((m + GJ_B - 1) / GJ_B) % 2 ? buf1 : buf0;
     cudaGetLastError();  // not launched: sweep launch by launch instead
   }
+  const int nt = (m + GJ_T - 1) / GJ_T;
   for (int k0 = 0; k0 < m; k0 += GJ_B) {
     k_gj_block<<<dim3(nt, nt), GJ_NT, 0, st>>>(a, b, m, k0, m - k0 < GJ_B ? m - k0 : GJ_B,
                                               status);
