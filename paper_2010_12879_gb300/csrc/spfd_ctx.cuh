@@ -169,18 +169,14 @@ struct spfd_ctx {
   // -G^T M a_cur; scratch of spfd_energy_grad (allocated on first use)
   const double *gJ_cur = nullptr;
   double *ev_stage = nullptr, *gj_stage = nullptr, *lam_stage = nullptr;
-  // scratch of spfd_percentile (allocated on first use, grown on demand):
-  // per-group counters, digit histograms, the key segments, the chunk table
-  // and its pinned host staging
-  unsigned long long *pct_small = nullptr, *pct_keys = nullptr, *pct_cand = nullptr,
-                     *pct_boff = nullptr;
-  unsigned *pct_hist = nullptr, *pct_bcnt = nullptr;
-  int *pct_candg = nullptr;
-  long long *pct_chunks = nullptr, *pct_hstage = nullptr;
-  long long pct_bcap = 0;
-  int pct_gcap = 0, pct_chcap = 0;
+  // scratch of spfd_percentile (allocated on first use, grown on demand): the
+  // first digit's table, the later digits', the groups with their pinned
+  // mirror, and the listed keys with their groups
+  unsigned *pct_first = nullptr, *pct_hist = nullptr;
+  unsigned long long *pct_grp = nullptr, *pct_hgrp = nullptr, *pct_keys = nullptr;
+  int *pct_keyg = nullptr;
+  int pct_gcap = 0;
   long long pct_keycap = 0, pct_nc = 0;  // pct_nc: conducting voxels seen last call
-  size_t pct_hstage_n = 0;
   // block orders chosen by the autotuner for batched launches: per batch
   // size, TF_COUNT x (levels) entries of 0 or 1; ord points at the table of
   // the batched solve in progress (nullptr: order 0 everywhere)
