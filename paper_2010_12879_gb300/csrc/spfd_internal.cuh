@@ -201,6 +201,49 @@ __device__ __forceinline__ bool f64_nonzero(double x) { return (f64_bits(x) << 1
 __device__ __forceinline__ bool f64_nonfinite(double x) {
   return ((f64_bits(x) >> 52) & 0x7ffull) == 0x7ffull;
 }
+// Correctly rounded square root of x, off the FP64 pipe (an FP64 sqrt takes a
+// dozen slots of it, 16 clocks each).  Integer square root by Newton's
+// iteration with an exact remainder (Zimmermann, "Karatsuba Square Root",
+// INRIA RR-3805, section 2, gives the remainder form): with x = N 4^k, N an
+// integer in [2^104, 2^106), the result's significand is the integer S nearest
+// to sqrt(N), and S is nearest exactly when -S < N - S^2 <= S (no ties: N -
+// S^2 is an integer, the midpoints are at S + 1/4).
+//   1. a 24-bit root from an FP32 reciprocal root (relative error at most
+//      2^-22) and one FP32 Newton step, relative error below 2^-22.9 with the
+//      truncation of N to 24 bits;
+//   2. a step with the remainder of the top 64 bits, N >> 42, in FP32: error
+//      below 2^-45, so that N - S^2 fits 62 bits and a sign;
+//   3. a step with the exact remainder, computed modulo 2^64: within one of
+//      the nearest; the final remainder decides.
+// Zero, subnormal, infinite, NaN and negative x go to sqrt().
+__device__ __forceinline__ double sqrt_rn(double x) {
+  const unsigned long long u = f64_bits(x);
+  const unsigned e = (unsigned)(u >> 52);  // sign and exponent
+  if (e - 1u >= 0x7feu) return sqrt(x);
+  const unsigned odd = ~e & 1u;  // the unbiased exponent is odd
+  // N = m 2^(52 + odd); f = N 2^-104 truncated to 24 bits, in [1, 4)
+  const unsigned long long m = (u & ((1ull << 52) - 1ull)) | (1ull << 52);
+  const float f = __uint_as_float(((127u + odd) << 23) | ((unsigned)(m >> 29) & 0x7fffffu));
+  const float y = rsqrtf(f);
+  float s = f * y;
+  s = fmaf(fmaf(-s, s, f), 0.5f * y, s);                 // in [1, 2]
+  const unsigned sh = (unsigned)(s * 2147483648.0f);     // S >> 21, in [2^31, 2^32)
+  const unsigned long long nh = m << (10 + odd);         // N >> 42
+  const long long r0 = (long long)(nh - (unsigned long long)sh * sh);
+  // r0 2^21 / (2 sh) = r0 y 2^-11, y being 2^31 / sh to 22 bits
+  const int d0 = __float2int_rn((float)(int)(r0 >> 14) * (y * 8.0f));
+  const unsigned long long S1 = ((unsigned long long)sh << 21) + (long long)d0;
+  const long long r1 = (long long)((m << (52 + odd)) - S1 * S1);
+  // r1 / (2 S1) = r1 y 2^-53
+  const int d1 = __float2int_rn((float)(int)(r1 >> 32) * (y * 0x1p-21f));
+  unsigned long long S = S1 + (long long)d1;
+  const long long r = r1 - (long long)d1 * (long long)(2 * S1 + (long long)d1);
+  if (r > (long long)S) ++S;
+  else if (r <= -(long long)S) --S;
+  // exponent (e - 1023 - odd) / 2 + 1023; a carry out of S moves into it
+  const unsigned re = (e - 1023u - odd + 2046u) >> 1;
+  return __longlong_as_double((long long)(((unsigned long long)(re - 1u) << 52) + S));
+}
 // w > 0 for a non-negative weight w: a bit test in FP64, a comparison in FP32.
 template <typename T>
 __device__ __forceinline__ bool weight_pos(T w) {
