@@ -636,14 +636,14 @@ k_energy(const unsigned char *__restrict__ mask, const double *__restrict__ a,
   }
 }
 
-// gJ_e = sum over the conducting voxels v at edge e of 2 c E_v,d(e) / Nc,
+// gJ_e = sum over the conducting voxels v at edge e of (2 c / Nc) E_v,d(e),
 // in increasing voxel order; one thread per node and direction.
 __global__ void __launch_bounds__(NT)
 k_energy_gJ(const unsigned char *__restrict__ mask, const double *__restrict__ Ev,
             int nx, int ny, int nz, double c, const Scalars *sc, double *__restrict__ gJ) {
   const size_t nv = (size_t)nx * ny * nz;
   const size_t NX = (size_t)nx + 1, NY = (size_t)ny + 1, NN = NX * NY * ((size_t)nz + 1);
-  const double nc = sc->aux[7];
+  const double nc = sc->aux[7], f = nc > 0.0 ? 2.0 * c / nc : 0.0;
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < 3 * NN;
        q += (size_t)gridDim.x * blockDim.x) {
     const int d = (int)(q / NN);
@@ -663,7 +663,7 @@ k_energy_gJ(const unsigned char *__restrict__ mask, const double *__restrict__ E
         else { vi += p1; vj += p2; }
         if (vi < 0 || vj < 0 || vk < 0 || vi >= nx || vj >= ny || vk >= nz) continue;
         const size_t v = ((size_t)vk * ny + vj) * nx + vi;
-        if (mask[v]) acc += 2.0 * c * Ev[d * nv + v] / nc;
+        if (mask[v]) acc += f * Ev[d * nv + v];
       }
     }
     gJ[q] = acc;
