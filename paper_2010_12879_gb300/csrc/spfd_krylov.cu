@@ -788,11 +788,17 @@ k_power27_f32(Grid g, const float *__restrict__ st, const float *__restrict__ di
     tile_full<float>(tl, v, bk, sn);
     __syncthreads();
     const size_t s = (size_t)bk * BV + t;
-    const float av = apply27_tile<float>(tl, st, S, s, t);
-    const float vs = tile_at(tl, t);
-    w[s] = dinv[s] * av;
-    two_sum_add(hi[0], lo[0], vs * av, 0.f);
-    two_sum_add(hi[1], lo[1], vs * vs * st[13 * S + s], 0.f);
+    // a clear activity bit: the row is zero, and so are v and w there
+    const bool on = (act_word(g, bk) >> (t & 31)) & 1u;
+    float wv = 0.f;
+    if (on) {
+      const float av = apply27_tile<float>(tl, st, S, s, t);
+      const float vs = tile_at(tl, t);
+      wv = dinv[s] * av;
+      two_sum_add(hi[0], lo[0], vs * av, 0.f);
+      two_sum_add(hi[1], lo[1], vs * vs * st[13 * S + s], 0.f);
+    }
+    w[s] = wv;
   }
   double tot[2];
   if (grid_sum_f32<2>(hi, lo, partials, &sc->ticket[4], tot, blockIdx.x, gridDim.x)) {
