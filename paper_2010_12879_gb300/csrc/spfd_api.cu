@@ -232,14 +232,14 @@ spfd_status project(spfd_ctx *c, T *v, int nk, int j0) {
     SPFD_LAUNCH(c, "project", f32, 3, 2 * (w + 4) * S, 12 * S,
                 launch_comp_sum<T>(l0.g.nb, v, c->comp, csum, c->ncomp, c->cstride, st, nk));
     SPFD_LAUNCH(c, "project", f32, 1, (2 * w + 4) * S, S,
-                launch_sub_mean<T>(l0.g.nb, v, c->comp, sc, 0, csum, c->csize, inv, st, nk,
+                launch_sub_mean<T>(l0.g.nb, v, c->ubits, c->comp, sc, 0, csum, c->csize, inv, st, nk,
                                    c->cstride));
   } else {
     SPFD_LAUNCH(c, "project", f32, 1, (w + 4) * S, S,
-                launch_dot<T>(l0.g.nb, v, nullptr, c->comp, sc, partials, 0, st, nk,
+                launch_dot<T>(l0.g.nb, v, nullptr, c->ubits, sc, partials, 0, st, nk,
                               c->pstride));
     SPFD_LAUNCH(c, "project", f32, 1, (2 * w + 4) * S, S,
-                launch_sub_mean<T>(l0.g.nb, v, c->comp, sc, 0, nullptr, c->csize, inv, st, nk));
+                launch_sub_mean<T>(l0.g.nb, v, c->ubits, c->comp, sc, 0, nullptr, c->csize, inv, st, nk));
   }
   return launch_check("projection");
 }
@@ -578,7 +578,7 @@ static spfd_status true_residual(spfd_ctx *c, const double *bb, double *rel, int
               (launch_residual7<double, double>(l0.g, l0.gx, l0.diag, c->xk, c->bk, l0.r,
                                                 c->stream, nk)));
   SPFD_LAUNCH(c, "true_residual", false, 1, 20 * S, 2 * S,
-              launch_dot<double>(l0.g.nb, l0.r, l0.r, c->comp, c->sc, c->partials, 2,
+              launch_dot<double>(l0.g.nb, l0.r, l0.r, c->ubits, c->sc, c->partials, 2,
                                  c->stream, nk, c->pstride));
   TRY(launch_check("true residual"));
   TRY(read_scalars(c, nk));
@@ -610,7 +610,7 @@ spfd_status precondition_step(spfd_ctx *c, T *r, T *p, int first, int nk, bool h
     SPFD_LAUNCH(c, "project", f32, 3, 2 * (w + 4) * S, 12 * S,
                 launch_comp_sum<T>(nb, z, c->comp, c->csum, c->ncomp, c->cstride, st, nk));
   SPFD_LAUNCH(c, "pupdate", f32, 1, (3 * w + 4) * S, 3 * S,
-              launch_pupdate<T>(nb, p, z, c->comp, c->sc, csum, c->csize, inv, st, nk,
+              launch_pupdate<T>(nb, p, z, c->ubits, c->comp, c->sc, csum, c->csize, inv, st, nk,
                                 c->cstride));
   return launch_check("V-cycle");
 }
@@ -662,12 +662,22 @@ static spfd_status vcycle_head(spfd_ctx *c, T *r, int nk) {
 // kernels on the stream, where a copy and an event cost 10 to 15 us an
 // iteration.  The stream is queried now and then, so that a failed launch
 // ends the wait.
+static double host_rr(const HostFlag &h) {
+  const unsigned long long u = (h.hi >> 32 << 32) | (h.lo >> 32);
+  double v;
+  memcpy(&v, &u, sizeof v);
+  return v;
+}
 static spfd_status wait_update(spfd_ctx *c, int na, const std::vector<int> &done) {
   auto t0 = std::chrono::steady_clock::now();
   for (int j = 0; j < na; ++j) {
     if (done[j]) continue;
     const HostFlag *h = c->hflag + j;
-    for (unsigned spins = 1; __atomic_load_n(&h->seq, __ATOMIC_ACQUIRE) != c->seq; ++spins) {
+    auto here = [&] {
+      return (unsigned)__atomic_load_n(&h->hi, __ATOMIC_ACQUIRE) == c->seq &&
+             (unsigned)__atomic_load_n(&h->lo, __ATOMIC_ACQUIRE) == c->seq;
+    };
+    for (unsigned spins = 1; !here(); ++spins) {
       if (spins % 256) continue;
       const auto t1 = std::chrono::steady_clock::now();
       if (t1 - t0 < std::chrono::milliseconds(1)) continue;
@@ -676,7 +686,7 @@ static spfd_status wait_update(spfd_ctx *c, int na, const std::vector<int> &done
       if (e == cudaErrorNotReady) continue;
       if (e != cudaSuccess)
         return fail(SPFD_ECUDA, "reading solver scalars: %s", cudaGetErrorString(e));
-      if (__atomic_load_n(&h->seq, __ATOMIC_ACQUIRE) != c->seq)
+      if (!here())
         return fail(SPFD_EINTERNAL, "the x / r update did not report its residual");
     }
   }
@@ -773,7 +783,7 @@ static spfd_status pcg(spfd_ctx *c, T *x, T *r, T *p, T *q, const T *opgx,
       if (done[j]) continue;
       res[j].iters = it;
       const double tol = tolv[j];
-      const double rrel = std::sqrt(c->hflag[j].rr / bb[j]);
+      const double rrel = std::sqrt(host_rr(c->hflag[j]) / bb[j]);
       last[1] = last[0];
       last[0] = rrel;
       if (!std::isfinite(rrel) || rrel > 1e8 * std::max(min_rrel[j], tol)) {
@@ -836,7 +846,7 @@ static spfd_status prepare_rhs(spfd_ctx *c, const double *a_dev, double *bb, int
   TRY(launch_check("rhs"));
   TRY(project<double>(c, c->bk, nk));
   SPFD_LAUNCH(c, "project", false, 1, 20 * S, 2 * S,
-              launch_dot<double>(l0.g.nb, c->bk, c->bk, c->comp, c->sc, c->partials, 1,
+              launch_dot<double>(l0.g.nb, c->bk, c->bk, c->ubits, c->sc, c->partials, 1,
                                  c->stream, nk, c->pstride));
   TRY(read_scalars(c, nk));
   if (c->hsc[0].status & DEV_BAD_A)  // one flag for the whole batch
@@ -931,7 +941,7 @@ static spfd_status solve_mixed(spfd_ctx *c, double tol, spfd_info *out, int nk =
                                       c->partials + (size_t)j * c->pstride, st));
     }
     SPFD_LAUNCH(c, "project", true, 1, 12 * S * na, 2 * S * na,
-                launch_dot<float>(nb, c->rk32, c->rk32, c->comp, c->sc, c->partials, 3, st,
+                launch_dot<float>(nb, c->rk32, c->rk32, c->ubits, c->sc, c->partials, 3, st,
                                   na, c->pstride));
     TRY(read_scalars(c, na));
     for (int j = 0; j < na; ++j) {
@@ -973,7 +983,7 @@ static spfd_status solve_mixed(spfd_ctx *c, double tol, spfd_info *out, int nk =
       TRY(project<double>(c, c->rk + (size_t)j * S0, 1, j));
       SPFD_LAUNCH(c, "project", false, 1, 20 * S, 2 * S,
                   launch_dot<double>(nb, c->rk + (size_t)j * S0, c->rk + (size_t)j * S0,
-                                     c->comp, c->sc + j, c->partials + (size_t)j * c->pstride,
+                                     c->ubits, c->sc + j, c->partials + (size_t)j * c->pstride,
                                      3, st));
       more = true;
     }

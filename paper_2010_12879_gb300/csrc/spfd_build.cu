@@ -525,6 +525,7 @@ spfd_status build_impl(spfd_ctx *c, const double *sigma) {
     // follows runs on the main stream after it
     TRY(dalloc(c, &parent, S0));
     TRY(dalloc(c, &c->comp, S0));
+    TRY(dalloc(c, &c->ubits, (size_t)std::max(nb0, 1) * 16));
     TRY(dalloc(c, &counts, nb0));
     TRY(dalloc(c, &offsets, nb0));
     TRY(halloc(c, &comp_hcnt, std::max(nb0, 1)));
@@ -678,7 +679,7 @@ spfd_status build_impl(spfd_ctx *c, const double *sigma) {
     SPFD_LAUNCH(c, "setup_components", false, 2, 0, 0, launch_assign_comp(l0.g, parent, offsets, c->comp, st));
     TRY(dalloc(c, &c->csize, std::max(c->ncomp, 1)));
     CU(cudaMemsetAsync(c->csize, 0, std::max(c->ncomp, 1) * sizeof(int), st));
-    SPFD_LAUNCH(c, "setup_components", false, 1, 0, 0, launch_comp_sizes(l0.g, c->comp, c->csize, st));
+    SPFD_LAUNCH(c, "setup_components", false, 1, 0, 0, launch_comp_sizes(l0.g, c->comp, c->csize, c->ubits, st));
     TRY(launch_check("component sizes"));
     dfree(c, parent);
     dfree(c, counts);

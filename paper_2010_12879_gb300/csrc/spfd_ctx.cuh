@@ -136,6 +136,7 @@ struct spfd_ctx {
   // fine-level bookkeeping
   unsigned char *mask = nullptr;  // [nz][ny][nx] conducting voxel flags
   int *comp = nullptr;            // [S0] component id or -1
+  unsigned *ubits = nullptr;      // [nb0][16] bits of the unknowns (comp >= 0)
   int ncomp = 0;
   int64_t ndof = 0;
   int *csize = nullptr;           // [ncomp]

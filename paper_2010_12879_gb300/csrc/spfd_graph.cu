@@ -313,7 +313,7 @@ spfd_status enqueue_true_residual(spfd_ctx *c) {
               (launch_residual7<double, double>(l0.g, l0.gx, l0.diag, c->xk, c->bk, l0.r,
                                                 c->stream, 1)));
   SPFD_LAUNCH(c, "true_residual", false, 1, 20 * S, 2 * S,
-              launch_dot<double>(l0.g.nb, l0.r, l0.r, c->comp, c->sc, c->partials, 2,
+              launch_dot<double>(l0.g.nb, l0.r, l0.r, c->ubits, c->sc, c->partials, 2,
                                  c->stream, 1, c->pstride));
   return launch_check("true residual");
 }
@@ -340,7 +340,7 @@ spfd_status capture_solve_fp64(spfd_ctx *c, GraphCtl *ctl, const double *a, doub
   TRY(last_node(s0, rhs_node));
   TRY(project<double>(c, c->bk, 1, 0));
   SPFD_LAUNCH(c, "project", false, 1, 20 * S, 2 * S,
-              launch_dot<double>(nb, c->bk, c->bk, c->comp, c->sc, c->partials, 1, s0, 1,
+              launch_dot<double>(nb, c->bk, c->bk, c->ubits, c->sc, c->partials, 1, s0, 1,
                                  c->pstride));
   CU(cudaMemsetAsync(c->xk, 0, S0 * sizeof(double), s0));
   CU(cudaMemcpyAsync(c->rk, c->bk, S0 * sizeof(double), cudaMemcpyDeviceToDevice, s0));
@@ -440,7 +440,7 @@ spfd_status capture_solve_mixed(spfd_ctx *c, GraphCtl *ctl, const double *a, dou
   TRY(last_node(s0, rhs_node));
   TRY(project<double>(c, c->bk, 1, 0));
   SPFD_LAUNCH(c, "project", false, 1, 20 * S, 2 * S,
-              launch_dot<double>(nb, c->bk, c->bk, c->comp, c->sc, c->partials, 1, s0, 1,
+              launch_dot<double>(nb, c->bk, c->bk, c->ubits, c->sc, c->partials, 1, s0, 1,
                                  c->pstride));
   CU(cudaMemsetAsync(c->xk, 0, S0 * sizeof(double), s0));
   CU(cudaMemcpyAsync(c->rk, c->bk, S0 * sizeof(double), cudaMemcpyDeviceToDevice, s0));
@@ -465,7 +465,7 @@ spfd_status capture_solve_mixed(spfd_ctx *c, GraphCtl *ctl, const double *a, dou
                   launch_scale_to_f32(nb, c->rk, 0.0, c->rk32, c->sc, c->partials, s2,
                                       &ctl->inv_nr));
       SPFD_LAUNCH(c, "project", true, 1, 12 * S, 2 * S,
-                  launch_dot<float>(nb, c->rk32, c->rk32, c->comp, c->sc, c->partials, 3, s2,
+                  launch_dot<float>(nb, c->rk32, c->rk32, c->ubits, c->sc, c->partials, 3, s2,
                                     1, c->pstride));
       // the inner FP32 CG
       CU(cudaMemsetAsync(c->pk32, 0, S0 * sizeof(float), s2));
@@ -513,7 +513,7 @@ spfd_status capture_solve_mixed(spfd_ctx *c, GraphCtl *ctl, const double *a, dou
                            body[2]));
         TRY(project<double>(c, c->rk, 1, 0));
         SPFD_LAUNCH(c, "project", false, 1, 20 * S, 2 * S,
-                    launch_dot<double>(nb, c->rk, c->rk, c->comp, c->sc, c->partials, 3,
+                    launch_dot<double>(nb, c->rk, c->rk, c->ubits, c->sc, c->partials, 3,
                                        body[2], 1, c->pstride));
         k_mctl_nrm<<<1, 1, 0, body[2]>>>(ctl, c->sc);
         TRY(launch_check("control"));

@@ -408,11 +408,10 @@ struct Scalars {
 };
 
 // What the host reads of a CG iteration, in pinned host memory that the last
-// block of the x / r update writes: |r|^2, then the number of that update.
+// block of the x / r update writes: the upper and the lower half of |r|^2,
+// each above the number of that update.
 struct HostFlag {
-  double rr;
-  unsigned seq;
-  unsigned pad;
+  unsigned long long hi, lo;
 };
 
 enum : int {
@@ -484,7 +483,9 @@ void launch_set_f64(double *p, double v, cudaStream_t st);
 void launch_brick_nbr(const Grid &g, int *nbr, cudaStream_t st);
 void launch_brick_kid(const Grid &gf, const Grid &gc, int *kid, cudaStream_t st);
 void launch_brick_par(const Grid &gf, const Grid &gc, int *par, cudaStream_t st);
-void launch_comp_sizes(const Grid &g, const int *comp, int *sizes,
+// Component sizes, and the unknowns' bits ([nb][16], bit t of word w: slot
+// b * 512 + 32 w + t is an unknown).
+void launch_comp_sizes(const Grid &g, const int *comp, int *sizes, unsigned *ubits,
                        cudaStream_t st);
 // Multigrid hierarchy (spfd_hierarchy.cu).  Pc: the fine level's compact
 // per-cell interpolation weights, [27][S/8] (row pc_off(q) + j, column
@@ -627,15 +628,15 @@ template <typename T>
 void launch_comp_sum(int nb, const T *v, const int *comp, double *ws, int ncomp,
                      int cstride, cudaStream_t st, int nk = 1);
 template <typename T>
-void launch_pupdate(int nb, T *p, const T *z, const int *comp,
+void launch_pupdate(int nb, T *p, const T *z, const unsigned *ubits, const int *comp,
                     const Scalars *sc, const double *csum, const int *csize,
                     double inv_ndof, cudaStream_t st, int nk = 1, int cstride = 0);
 template <typename T>
-void launch_sub_mean(int nb, T *v, const int *comp, const Scalars *sc,
+void launch_sub_mean(int nb, T *v, const unsigned *ubits, const int *comp, const Scalars *sc,
                      int aux_slot, const double *csum, const int *csize,
                      double inv_ndof, cudaStream_t st, int nk = 1, int cstride = 0);
 template <typename T>
-void launch_dot(int nb, const T *x, const T *y, const int *comp, Scalars *sc,
+void launch_dot(int nb, const T *x, const T *y, const unsigned *ubits, Scalars *sc,
                 double *partials, int slot, cudaStream_t st, int nk = 1, size_t pstride = 0);
 template <typename T>
 void launch_scatter(const Grid &g, const T *x, const int *comp, double *psi,

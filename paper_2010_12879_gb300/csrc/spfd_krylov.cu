@@ -177,16 +177,16 @@ k_update_xr(int nb, T *__restrict__ x, T *__restrict__ r,
   const Acc<T> v[2] = {rr, rs_sum};
   double tot[2];
   if (grid_sum_acc<T, 2>(v, partials, &sc->ticket[1], tot, blockIdx.x, gridDim.x)) {
-    if (hf) {  // r.r before its number: the host reads them in the other order
-      volatile HostFlag *h = hf + blockIdx.y;
-      h->rr = tot[0];
-      __threadfence_system();
-      h->seq = seq;
-    }
     sc->rr = tot[0];
     sc->rsum = tot[1];
     sc->rmean = tot[1] * sc->inv_ndof;
     sc->rmean_f = (float)sc->rmean;
+    if (hf) {  // each word carries the number, so no fence orders the two
+      const unsigned long long u = (unsigned long long)__double_as_longlong(tot[0]);
+      volatile HostFlag *h = hf + blockIdx.y;
+      h->hi = (u >> 32 << 32) | seq;
+      h->lo = (u << 32) | seq;
+    }
   }
 }
 
@@ -322,11 +322,18 @@ __global__ void k_comp_finish(double *ws, int cstride, int ncomp) {
   ws[c] = scalbn(neg ? -mag : mag, -sum_scale_exp(mb));
 }
 
-// p = (z - mean_c(z)) + beta p on the unknowns.  One component: the mean is
-// sc->zmean; several: csum[c] / csize[c].
-template <typename T>
+// The unknown bits of the N consecutive slots from s0 on (N divides 32).
+template <int N>
+__device__ __forceinline__ unsigned unknown_bits(const unsigned *__restrict__ ubits, size_t s0) {
+  return (__ldg(&ubits[s0 >> 5]) >> (s0 & 31)) & ((1u << N) - 1u);
+}
+
+// p = (z - mean_c(z)) + beta p on the unknowns.  One component (csum null):
+// the mean is sc->zmean, and the unknowns come from their bits, an eighth of
+// a byte a slot instead of the four of comp; several: csum[c] / csize[c].
+template <typename T, bool MULTI>
 __global__ void __launch_bounds__(NT)
-k_pupdate(T *__restrict__ p, const T *__restrict__ z,
+k_pupdate(T *__restrict__ p, const T *__restrict__ z, const unsigned *__restrict__ ubits,
           const int *__restrict__ comp, const Scalars *sc,
           const double *__restrict__ csum, const int *__restrict__ csize, int cstride) {
   pdl_entry();
@@ -336,64 +343,83 @@ k_pupdate(T *__restrict__ p, const T *__restrict__ z,
     const size_t off = (size_t)blockIdx.y * gridDim.x * BV;
     p += off; z += off;
     sc += blockIdx.y;
-    if (csum) csum += (size_t)blockIdx.y * cstride;
+    if (MULTI) csum += (size_t)blockIdx.y * cstride;
   }
   T mean1, beta;
   if constexpr (sizeof(T) == 4) { mean1 = sc->zmean_f; beta = sc->beta_f; }
   else { mean1 = sc->zmean; beta = sc->beta; }
+  const unsigned on = unknown_bits<N>(ubits, s0);
   int c[N];
-  ld_ints<N>(comp + s0, c);
+  if (MULTI) ld_ints<N>(comp + s0, c);
   const V16<T> zv = ld16(z + s0);
   V16<T> pv = ld16(p + s0);
 #pragma unroll
   for (int i = 0; i < N; ++i) {
-    if (c[i] < 0) { pv.v[i] = (T)0; continue; }
-    const T mean = csum ? (T)(csum[c[i]] / (double)csize[c[i]]) : mean1;
+    if (!((on >> i) & 1u)) { pv.v[i] = (T)0; continue; }
+    const T mean = MULTI ? (T)(csum[c[i]] / (double)csize[c[i]]) : mean1;
     pv.v[i] = (zv.v[i] - mean) + beta * pv.v[i];
   }
   st16(p + s0, pv);
 }
 
-// v -= mean_c(v) on the unknowns (single component: mean = aux[slot] / n).
-template <typename T>
+// v -= mean_c(v) on the unknowns, 0 elsewhere (single component: mean =
+// aux[slot] / n).
+template <typename T, bool MULTI>
 __global__ void __launch_bounds__(NT)
-k_sub_mean(T *__restrict__ v, const int *__restrict__ comp, const Scalars *sc,
-           int aux_slot, const double *__restrict__ csum,
+k_sub_mean(T *__restrict__ v, const unsigned *__restrict__ ubits, const int *__restrict__ comp,
+           const Scalars *sc, int aux_slot, const double *__restrict__ csum,
            const int *__restrict__ csize, int cstride) {
   pdl_entry();
-  const size_t s = (size_t)blockIdx.x * BV + threadIdx.x;
+  constexpr int N = V16<T>::N;
+  const size_t s0 = (size_t)blockIdx.x * BV + threadIdx.x * N;
   v += (size_t)blockIdx.y * gridDim.x * BV;
   sc += blockIdx.y;
-  if (csum) csum += (size_t)blockIdx.y * cstride;
-  const int c = comp[s];
-  if (c < 0) { v[s] = (T)0; return; }
-  const T mean = csum ? (T)(csum[c] / (double)csize[c])
-                      : (T)(sc->aux[aux_slot] * sc->inv_ndof);
-  v[s] = v[s] - mean;
+  if (MULTI) csum += (size_t)blockIdx.y * cstride;
+  const unsigned on = unknown_bits<N>(ubits, s0);
+  int c[N];
+  if (MULTI) ld_ints<N>(comp + s0, c);
+  const T mean1 = (T)(sc->aux[aux_slot] * sc->inv_ndof);
+  V16<T> x = ld16(v + s0);
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const T mean =
+        MULTI && ((on >> i) & 1u) ? (T)(csum[c[i]] / (double)csize[c[i]]) : mean1;
+    x.v[i] = ((on >> i) & 1u) ? x.v[i] - mean : (T)0;
+  }
+  st16(v + s0, x);
 }
 
 // aux[slot] = sum over unknowns of x*y (y = null: plain sum of x).
-template <typename T>
+// A thread adds its slot of bricks blockIdx.x, + gridDim.x, ... in turn; x.x
+// reads x once.
+template <typename T, bool PROD>
 __global__ void __launch_bounds__(NT)
 k_dot(int nb, const T *__restrict__ x, const T *__restrict__ y,
-      const int *__restrict__ comp, Scalars *sc, double *partials, int slot,
+      const unsigned *__restrict__ ubits, Scalars *sc, double *partials, int slot,
       size_t pstride) {
   pdl_entry();
+  const bool square = PROD && x == y;
   {
     const size_t off = (size_t)blockIdx.y * nb * BV;
     x += off;
-    if (y) y += off;
+    if (PROD) y += off;
     sc += blockIdx.y;
     partials += (size_t)blockIdx.y * pstride;
   }
   Acc<T> acc;
+  const int t = threadIdx.x;
   for (int bk = blockIdx.x; bk < nb; bk += gridDim.x) {
-    const size_t s = (size_t)bk * BV + threadIdx.x;
-    if (comp[s] >= 0) acc.add(y ? x[s] * y[s] : x[s]);
+    const size_t s = (size_t)bk * BV + t;
+    const T xv = x[s], yv = PROD && !square ? y[s] : xv;
+    if ((__ldg(&ubits[(size_t)bk * 16 + (t >> 5)]) >> (t & 31)) & 1u) {
+      if (PROD) acc.add(xv * yv);
+      else acc.add(xv);
+    }
   }
   const Acc<T> v[1] = {acc};
   double tot[1];
-  if (grid_sum_acc<T, 1>(v, partials, &sc->ticket[3], tot, blockIdx.x, gridDim.x)) sc->aux[slot] = tot[0];
+  if (grid_sum_acc<T, 1>(v, partials, &sc->ticket[3], tot, blockIdx.x, gridDim.x))
+    sc->aux[slot] = tot[0];
 }
 
 // ------------------------------------------------------------ Eq. 3 RHS
@@ -875,14 +901,22 @@ __global__ void k_convert(size_t n, const double *__restrict__ src, double f,
   }
 }
 
-// x += f * d (FP64 accumulation of an FP32 correction) on level-0 slots.
-__global__ void __launch_bounds__(NT)
+// x += f * d (FP64 accumulation of an FP32 correction) on level-0 slots, four
+// per thread.
+__global__ void __launch_bounds__(BV / 4)
 k_axpy_mixed(double *__restrict__ x, const float *__restrict__ d, double f,
              const double *__restrict__ fdev) {
   pdl_entry();
   if (fdev) f = *fdev;
-  const size_t s = (size_t)blockIdx.x * BV + threadIdx.x;
-  x[s] += f * (double)d[s];
+  const size_t s = (size_t)blockIdx.x * BV + 4 * threadIdx.x;
+  const V16<float> dv = ld16(d + s);
+  V16<double> a = ld16(x + s), b = ld16(x + s + 2);
+  a.v[0] += f * (double)dv.v[0];
+  a.v[1] += f * (double)dv.v[1];
+  b.v[0] += f * (double)dv.v[2];
+  b.v[1] += f * (double)dv.v[3];
+  st16(x + s, a);
+  st16(x + s + 2, b);
 }
 
 // r32 = (float)(f * r64); sum(r32) and its mean land in sc->rsum / rmean_f
@@ -924,7 +958,7 @@ template void launch_convert<__nv_bfloat16>(size_t, const double *, double,
                                             __nv_bfloat16 *, cudaStream_t);
 void launch_axpy_mixed(int nb, double *x, const float *d, double f,
                        cudaStream_t st, const double *fdev) {
-  if (nb) pdl(k_axpy_mixed, nb, NT, st)(x, d, f, fdev);
+  if (nb) pdl(k_axpy_mixed, nb, BV / 4, st)(x, d, f, fdev);
 }
 void launch_scale_to_f32(int nb, const double *r, double f, float *r32,
                          Scalars *sc, double *partials, cudaStream_t st, const double *fdev) {
@@ -999,23 +1033,34 @@ void launch_comp_sum(int nb, const T *v, const int *comp, double *ws, int ncomp,
   pdl(k_comp_finish, dim3((ncomp + 255) / 256, nk), 256, st)(ws, cstride, ncomp);
 }
 template <typename T>
-void launch_pupdate(int nb, T *p, const T *z, const int *comp,
+void launch_pupdate(int nb, T *p, const T *z, const unsigned *ubits, const int *comp,
                     const Scalars *sc, const double *csum, const int *csize,
                     double, cudaStream_t st, int nk, int cstride) {
-  if (nb) pdl(k_pupdate<T>, dim3(nb, nk), NT / V16<T>::N, st)(p, z, comp, sc, csum, csize, cstride);
+  if (!nb) return;
+  const dim3 grid(nb, nk), block(NT / V16<T>::N);
+  if (csum)
+    pdl(k_pupdate<T, true>, grid, block, st)(p, z, ubits, comp, sc, csum, csize, cstride);
+  else
+    pdl(k_pupdate<T, false>, grid, block, st)(p, z, ubits, comp, sc, csum, csize, cstride);
 }
 template <typename T>
-void launch_sub_mean(int nb, T *v, const int *comp, const Scalars *sc,
+void launch_sub_mean(int nb, T *v, const unsigned *ubits, const int *comp, const Scalars *sc,
                      int aux_slot, const double *csum, const int *csize,
                      double, cudaStream_t st, int nk, int cstride) {
-  if (nb) pdl(k_sub_mean<T>, dim3(nb, nk), NT, st)(v, comp, sc, aux_slot, csum, csize, cstride);
+  if (!nb) return;
+  const dim3 grid(nb, nk), block(NT / V16<T>::N);
+  if (csum)
+    pdl(k_sub_mean<T, true>, grid, block, st)(v, ubits, comp, sc, aux_slot, csum, csize, cstride);
+  else
+    pdl(k_sub_mean<T, false>, grid, block, st)(v, ubits, comp, sc, aux_slot, csum, csize, cstride);
 }
 template <typename T>
-void launch_dot(int nb, const T *x, const T *y, const int *comp, Scalars *sc,
+void launch_dot(int nb, const T *x, const T *y, const unsigned *ubits, Scalars *sc,
                 double *partials, int slot, cudaStream_t st, int nk, size_t pstride) {
-  if (nb)
-    pdl(k_dot<T>, dim3(std::min(nb, RED_GRID), nk), NT, st)(nb, x, y, comp, sc, partials,
-                                                              slot, pstride);
+  if (!nb) return;
+  const dim3 grid(std::min(nb, RED_GRID), nk);
+  if (y) pdl(k_dot<T, true>, grid, NT, st)(nb, x, y, ubits, sc, partials, slot, pstride);
+  else pdl(k_dot<T, false>, grid, NT, st)(nb, x, y, ubits, sc, partials, slot, pstride);
 }
 void launch_rhs(const Grid &g, const double *gx, const double *a, double *b,
                 int *status, cudaStream_t st, int nk) {
@@ -1112,14 +1157,15 @@ void launch_energy_grads(const Grid &g, const double *gx, const unsigned char *m
                                  size_t);                                      \
   template void launch_comp_sum<T>(int, const T *, const int *, double *, int, \
                                    int, cudaStream_t, int);                    \
-  template void launch_pupdate<T>(int, T *, const T *, const int *,            \
-                                  const Scalars *, const double *,             \
-                                  const int *, double, cudaStream_t, int,      \
-                                  int);                                        \
-  template void launch_sub_mean<T>(int, T *, const int *, const Scalars *,     \
-                                   int, const double *, const int *, double,   \
-                                   cudaStream_t, int, int);                    \
-  template void launch_dot<T>(int, const T *, const T *, const int *,          \
+  template void launch_pupdate<T>(int, T *, const T *, const unsigned *,       \
+                                  const int *, const Scalars *,                \
+                                  const double *, const int *, double,         \
+                                  cudaStream_t, int, int);                     \
+  template void launch_sub_mean<T>(int, T *, const unsigned *, const int *,    \
+                                   const Scalars *, int, const double *,       \
+                                   const int *, double, cudaStream_t, int,     \
+                                   int);                                       \
+  template void launch_dot<T>(int, const T *, const T *, const unsigned *,     \
                               Scalars *, double *, int, cudaStream_t, int,     \
                               size_t);                                         \
   template void launch_scatter<T>(const Grid &, const T *, const int *,        \

@@ -399,10 +399,12 @@ void launch_assign_comp(const Grid &g, const int *parent, const int *offsets,
 }
 
 __global__ void __launch_bounds__(NT)
-k_comp_sizes(const int *__restrict__ comp, int *sizes) {
+k_comp_sizes(const int *__restrict__ comp, int *sizes, unsigned *__restrict__ ubits) {
   __shared__ int c0;
   const int s = blockIdx.x * BV + threadIdx.x;
   const int c = comp[s];
+  const unsigned word = __ballot_sync(0xffffffffu, c >= 0);
+  if ((threadIdx.x & 31) == 0) ubits[s >> 5] = word;
   // a brick inside one component (the common case) adds its count once
   if (threadIdx.x == 0) c0 = -1;
   __syncthreads();
@@ -419,10 +421,10 @@ k_comp_sizes(const int *__restrict__ comp, int *sizes) {
     atomicAdd(&sizes[c], __popc(grp));
 }
 
-void launch_comp_sizes(const Grid &g, const int *comp, int *sizes,
+void launch_comp_sizes(const Grid &g, const int *comp, int *sizes, unsigned *ubits,
                        cudaStream_t st) {
   if (g.nb == 0) return;
-  k_comp_sizes<<<g.nb, NT, 0, st>>>(comp, sizes);
+  k_comp_sizes<<<g.nb, NT, 0, st>>>(comp, sizes, ubits);
 }
 
 // Diagonal, its inverse, and the level's largest diagonal (for a relative
