@@ -517,7 +517,7 @@ k_gather(Grid g, const double *__restrict__ psi, const int *__restrict__ comp,
 // its x-edge terms at rows j and j+1 (X0, X1, with Psi of column i+1 from the
 // next lane) and its y-edge term (Y), and per voxel layer its two z-edge terms
 // (Z0, Z1); voxel i takes the y and z terms of column i+1 from the next lane
-// too.  Block y walks EF_KCHUNK voxel layers and carries the terms of layer
+// too.  Block y walks kchunk voxel layers and carries the terms of layer
 // k+1 into layer k+1's voxels, so a layer's terms are formed once.  Layers
 // with no conducting voxel in the warp form nothing (their voxels get 0).
 // Per voxel layer a column forms 5 terms (10 FP64 additions) against 16 when
@@ -526,10 +526,14 @@ k_gather(Grid g, const double *__restrict__ psi, const int *__restrict__ comp,
 // the kernel.  The root is taken off it (sqrt_rn, integer and FP32
 // instructions): 0.89 -> 0.70 ms on the 2 mm body.
 constexpr int EF_THREADS = 256;
-constexpr int EF_KCHUNK = 16;
 // 4 resident blocks per SM (at most 64 registers a thread): the kernel waits
 // on memory between layers, and the FP64 pipe needs the warps to cover it.
 constexpr int EF_MIN_BLOCKS = 4;
+// Layers a block walks: 16, halved while fewer than this many warps would
+// start (a small grid's time is the walk's dependent loads: 54 us for the 32^3
+// and 16 mm grids with 16 layers, 9 us now; the 4 mm body 171 -> 116 us; the
+// 2 mm body starts 74,000 warps with 16).
+constexpr long long EF_WARPS = 20000;
 
 struct EfTerms {
   double p0, p1;  // Psi(i, j, k), Psi(i, j+1, k)
@@ -559,7 +563,7 @@ __device__ __forceinline__ EfTerms ef_layer(const double *__restrict__ a,
 __global__ void __launch_bounds__(EF_THREADS, EF_MIN_BLOCKS)
 k_efield(const unsigned char *__restrict__ mask, const double *__restrict__ a,
          const double *__restrict__ psi, int nx, int ny, int nz, double c,
-         double *__restrict__ E) {
+         double *__restrict__ E, int kchunk) {
   const int lane = threadIdx.x & 31;
   const long long warp = ((long long)blockIdx.x * EF_THREADS + threadIdx.x) >> 5;
   const size_t NX = (size_t)nx + 1, NXY = NX * ((size_t)ny + 1);
@@ -571,7 +575,7 @@ k_efield(const unsigned char *__restrict__ mask, const double *__restrict__ a,
   const int i = live ? (int)(col % (long long)NX) : 0, j = live ? (int)(col / (long long)NX) : 0;
   const bool own = live && lane < 31 && i < nx;
   const size_t nc = (size_t)j * NX + i;
-  const int kb = blockIdx.y * EF_KCHUNK, ke = min(kb + EF_KCHUNK, nz);
+  const int kb = blockIdx.y * kchunk, ke = min(kb + kchunk, nz);
   EfTerms T{};
   bool have = false;  // T holds layer k's terms (warp-uniform)
   for (int k = kb; k < ke; ++k) {
@@ -1085,9 +1089,11 @@ void launch_efield(const unsigned char *mask, const double *a,
   if ((size_t)nx * ny * nz == 0) return;
   const long long ncol = (long long)(nx + 1) * ny;
   const long long warps = (ncol + 30) / 31;
+  int kchunk = 16;
+  while (kchunk > 1 && warps * ((nz + kchunk - 1) / kchunk) < EF_WARPS) kchunk /= 2;
   const dim3 grid((unsigned)((warps * 32 + EF_THREADS - 1) / EF_THREADS),
-                  (unsigned)((nz + EF_KCHUNK - 1) / EF_KCHUNK));
-  k_efield<<<grid, EF_THREADS, 0, st>>>(mask, a, psi, nx, ny, nz, omega / (4.0 * h), E);
+                  (unsigned)((nz + kchunk - 1) / kchunk));
+  k_efield<<<grid, EF_THREADS, 0, st>>>(mask, a, psi, nx, ny, nz, omega / (4.0 * h), E, kchunk);
 }
 
 // |E| of a complex source from the magnitudes of its real and imaginary
