@@ -176,7 +176,7 @@ __device__ __forceinline__ void interp_node(const LevelOp &A, double *__restrict
       }
       const double den = ac[13];
       if (den > 1e-12 * dg) {
-        const double inv = -1.0 / den;
+        const double inv = -recip_rn(den);
 #pragma unroll
         for (int r = 0; r < NW; ++r) w[r] = acc[r] * inv;
       } else {
@@ -198,8 +198,14 @@ template <int PASS>
 constexpr int interp_classes() { return PASS == 1 ? 4 : (PASS == 2 ? 3 : 1); }
 template <int PASS>
 constexpr int interp_bricks() { return PASS == 3 ? 8 : 2; }
+// Resident blocks asked for: the passes wait on scattered loads, and with one
+// block (60 to 90 registers) too few warps cover them.  2 mm body, level 0, us
+// per pass: 220 / 205 / 153 with one, 193 / 192 / 142 with two, 139 / 172 /
+// 134 with three, 113 / 170 / 139 with four (the last two columns also have
+// the reciprocal off the FP64 pipe); level 1: 82 / 74 / 83 with one, 65 / 73 /
+// 67 with two, 64 / 69 / 91 with three.
 template <bool K27, int PASS>
-__global__ void __launch_bounds__(NT) k_interp(LevelOp A, double *__restrict__ Pc) {
+__global__ void __launch_bounds__(NT, K27 ? 2 : (PASS == 1 ? 4 : 3)) k_interp(LevelOp A, double *__restrict__ Pc) {
   constexpr int NCL = interp_classes<PASS>();
   const int cell = threadIdx.x & 63, grp = threadIdx.x >> 6;
   const int ci = grp % NCL, b = blockIdx.x * interp_bricks<PASS>() + grp / NCL;
@@ -328,7 +334,8 @@ __device__ __forceinline__ void ptap_layer(const Grid &gf, const Grid &gc, size_
 
 // Each also writes the coarse level's activity bits (Grid::act): the bit of
 // a coarse node is set when one of its 27 weights P[d] is not zero.
-__global__ void __launch_bounds__(NT)
+// (Two resident blocks: 705 -> 660 us for level 1 of the 2 mm body.)
+__global__ void __launch_bounds__(NT, 2)
 k_ptap(Grid gf, Grid gc, size_t NCf, const double *__restrict__ Pc,
        const double *__restrict__ T, double *__restrict__ stc, double *__restrict__ P,
        unsigned *__restrict__ act) {

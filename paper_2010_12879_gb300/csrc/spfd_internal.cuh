@@ -244,6 +244,35 @@ __device__ __forceinline__ double sqrt_rn(double x) {
   const unsigned re = (e - 1023u - odd + 2046u) >> 1;
   return __longlong_as_double((long long)(((unsigned long long)(re - 1u) << 52) + S));
 }
+// Correctly rounded 1 / x, off the FP64 pipe in the manner of sqrt_rn: Newton's
+// iteration for the integer quotient with an exact remainder.  With x = m
+// 2^(e - 1075), m in [2^52, 2^53), the result's significand is the integer Q
+// nearest to 2^105 / m, which is the one with |2^105 - Q m| <= m / 2 (no
+// ties).  A 24-bit quotient comes from an FP32 reciprocal and one FP32 Newton
+// step (relative error below 2^-22.5 with the truncation of m to 24 bits); the
+// remainder 2^83 - qh m then fits 61 bits and is exact modulo 2^64, as is the
+// next one; the last remainder decides.  Zero, subnormal and huge x, infinity
+// and NaN take the division.
+__device__ __forceinline__ double recip_rn(double x) {
+  const unsigned long long u = f64_bits(x);
+  const unsigned e = (unsigned)(u >> 52) & 0x7ffu;
+  if (e - 1u >= 2043u) return 1.0 / x;
+  const long long m = (long long)((u & ((1ull << 52) - 1ull)) | (1ull << 52));
+  const float f = __uint_as_float((127u << 23) | ((unsigned)(m >> 29) & 0x7fffffu));
+  float y = __fdividef(1.0f, f);
+  y = fmaf(y, fmaf(-f, y, 1.0f), y);
+  const unsigned qh = (unsigned)(y * 2147483648.0f);  // Q >> 22
+  const long long r0 = -((long long)qh * m);           // 2^83 - qh m
+  const int d0 = __float2int_rn((float)(int)(r0 >> 30) * y);
+  const long long r1 = (r0 << 22) - (long long)d0 * m;
+  const int d1 = __float2int_rn((float)(int)(r1 >> 32) * (y * 0x1p-20f));
+  long long Q = ((long long)qh << 22) + d0 + d1;
+  const long long r = r1 - (long long)d1 * m;
+  if (2 * r > m) ++Q;
+  else if (2 * r < -m) --Q;
+  return __longlong_as_double(
+      (long long)((u & (1ull << 63)) | (((unsigned long long)(2044u - e) << 52) + Q)));
+}
 // w > 0 for a non-negative weight w: a bit test in FP64, a comparison in FP32.
 template <typename T>
 __device__ __forceinline__ bool weight_pos(T w) {
