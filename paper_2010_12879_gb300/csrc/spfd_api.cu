@@ -1091,7 +1091,7 @@ static spfd_status solve_device(spfd_ctx *c, const double *a_dev, double tol,
     TRY(s);
     const double NN = (double)NNs * nk;
     SPFD_LAUNCH(c, "scatter", false, 1, 8 * NN + 12.0 * l0.S * nk, 0,
-                launch_scatter<double>(l0.g, c->xk, c->comp, psi_dev, st, nk));
+                launch_scatter<double>(l0.g, c->xk, c->ubits, psi_dev, st, nk));
     TRY(launch_check("scatter"));
   }
   CU(cudaEventRecord(c->ev1, st));

@@ -301,7 +301,7 @@ spfd_status patch_ptr(cudaGraphExec_t ex, cudaGraphNode_t node, int nargs, int i
 }
 
 // Argument positions of the pointers patched per solve:
-// k_rhs(Grid, gx, a, b, status) and k_scatter<double>(Grid, x, comp, psi).
+// k_rhs(Grid, gx, a, b, status) and k_scatter<double>(Grid, x, ubits, psi).
 constexpr int RHS_NARGS = 5, RHS_ARG_A = 2;
 constexpr int SCATTER_NARGS = 4, SCATTER_ARG_PSI = 3;
 
@@ -416,7 +416,7 @@ spfd_status capture_solve_fp64(spfd_ctx *c, GraphCtl *ctl, const double *a, doub
   c->stream = s0;
   const double NN = (double)(c->nx + 1) * (c->ny + 1) * (c->nz + 1);
   SPFD_LAUNCH(c, "scatter", false, 1, 8 * NN + 12.0 * S, 0,
-              launch_scatter<double>(l0.g, c->xk, c->comp, psi, s0, 1));
+              launch_scatter<double>(l0.g, c->xk, c->ubits, psi, s0, 1));
   TRY(launch_check("scatter"));
   TRY(last_node(s0, scatter_node));
   return SPFD_OK;
@@ -529,7 +529,7 @@ spfd_status capture_solve_mixed(spfd_ctx *c, GraphCtl *ctl, const double *a, dou
   TRY(project<double>(c, c->xk, 1, 0));
   const double NN = (double)(c->nx + 1) * (c->ny + 1) * (c->nz + 1);
   SPFD_LAUNCH(c, "scatter", false, 1, 8 * NN + 12.0 * S, 0,
-              launch_scatter<double>(l0.g, c->xk, c->comp, psi, s0, 1));
+              launch_scatter<double>(l0.g, c->xk, c->ubits, psi, s0, 1));
   TRY(launch_check("scatter"));
   TRY(last_node(s0, scatter_node));
   return SPFD_OK;

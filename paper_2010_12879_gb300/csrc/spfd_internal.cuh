@@ -668,7 +668,7 @@ template <typename T>
 void launch_dot(int nb, const T *x, const T *y, const unsigned *ubits, Scalars *sc,
                 double *partials, int slot, cudaStream_t st, int nk = 1, size_t pstride = 0);
 template <typename T>
-void launch_scatter(const Grid &g, const T *x, const int *comp, double *psi,
+void launch_scatter(const Grid &g, const T *x, const unsigned *ubits, double *psi,
                     cudaStream_t st, int nk = 1);
 void launch_rhs(const Grid &g, const double *gx, const double *a, double *b,
                 int *status, cudaStream_t st, int nk = 1);

@@ -472,20 +472,30 @@ k_rhs(Grid g, const double *__restrict__ gx, const double *__restrict__ a,
   if (bad) atomicOr(status, DEV_BAD_A);
 }
 
+// Coordinates of entry n of an array nx x ny x ... (x fastest).  Node and
+// voxel counts are below 2^31 (spfd_build), so 32-bit divisions do; as 64-bit
+// ones they took more time than the rest of the kernels that use them.
+__device__ __forceinline__ void grid_ijk(unsigned n, int nx, int ny, int *i, int *j, int *k) {
+  const unsigned r = n / (unsigned)nx, q = r / (unsigned)ny;
+  *i = (int)(n - r * (unsigned)nx);
+  *j = (int)(r - q * (unsigned)ny);
+  *k = (int)q;
+}
+
 // psi[n] = x[slot(n)] on the full node grid (0 where no unknown).
 template <typename T>
 __global__ void k_scatter(Grid g, const T *__restrict__ x,
-                          const int *__restrict__ comp, double *__restrict__ psi) {
+                          const unsigned *__restrict__ ubits, double *__restrict__ psi) {
   pdl_entry();
   const size_t NN = (size_t)g.NX * g.NY * g.NZ;
   x += (size_t)blockIdx.y * g.nb * BV;
   psi += (size_t)blockIdx.y * NN;
   for (size_t n = blockIdx.x * (size_t)blockDim.x + threadIdx.x; n < NN;
        n += (size_t)gridDim.x * blockDim.x) {
-    const int i = (int)(n % g.NX), j = (int)((n / g.NX) % g.NY),
-              k = (int)(n / ((size_t)g.NX * g.NY));
+    int i, j, k;
+    grid_ijk((unsigned)n, g.NX, g.NY, &i, &j, &k);
     const int s = slot_at(g, i, j, k);
-    psi[n] = (s >= 0 && comp[s] >= 0) ? (double)x[s] : 0.0;
+    psi[n] = s >= 0 && unknown_bits<1>(ubits, s) ? (double)x[s] : 0.0;
   }
 }
 
@@ -617,13 +627,6 @@ k_efield(const unsigned char *__restrict__ mask, const double *__restrict__ a,
 // which the edge-conductance rule (g_e = h/4 * sum of the 4 voxels' sigma)
 // turns into dJ/dsigma_v = h/4 * sum over the voxel's 12 edges of dJ/dg.
 
-__device__ __forceinline__ void voxel_ijk(size_t v, int nx, int ny, int *i, int *j, int *k) {
-  const size_t r = v / (size_t)nx;
-  *i = (int)(v - r * nx);
-  *j = (int)(r % (size_t)ny);
-  *k = (int)(r / (size_t)ny);
-}
-
 // Ev[d][v] = E_v,d (0 in air); sc->aux[6] = sum |E_v|^2, sc->aux[7] = Nc.
 __global__ void __launch_bounds__(NT)
 k_energy(const unsigned char *__restrict__ mask, const double *__restrict__ a,
@@ -637,7 +640,7 @@ k_energy(const unsigned char *__restrict__ mask, const double *__restrict__ a,
     double E[3] = {0.0, 0.0, 0.0};
     if (mask[v]) {
       int i, j, k;
-      voxel_ijk(v, nx, ny, &i, &j, &k);
+      grid_ijk((unsigned)v, nx, ny, &i, &j, &k);
       const size_t n = (size_t)k * NXY + (size_t)j * NX + i;
 #pragma unroll
       for (int st = 0; st < 4; ++st) {  // (s, t) = (0,0), (0,1), (1,0), (1,1)
@@ -676,9 +679,10 @@ k_energy_gJ(const unsigned char *__restrict__ mask, const double *__restrict__ E
   const double nc = sc->aux[7], f = nc > 0.0 ? 2.0 * c / nc : 0.0;
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < 3 * NN;
        q += (size_t)gridDim.x * blockDim.x) {
-    const int d = (int)(q / NN);
+    const int d = (q >= NN) + (q >= 2 * NN);
     const size_t n = q - (size_t)d * NN;
-    const int i = (int)(n % NX), j = (int)((n / NX) % NY), k = (int)(n / (NX * NY));
+    int i, j, k;
+    grid_ijk((unsigned)n, nx + 1, ny + 1, &i, &j, &k);
     double acc = 0.0;
     // the up to 4 voxels at the edge, lowest voxel index first: offsets on
     // the two axes other than d, (-1,-1), (0,-1), (-1,0), (0,0)
@@ -732,7 +736,8 @@ k_energy_grad_a(Grid g, const double *__restrict__ gx, const double *__restrict_
   const size_t S = (size_t)g.nb * BV;
   for (size_t n = blockIdx.x * (size_t)blockDim.x + threadIdx.x; n < NN;
        n += (size_t)gridDim.x * blockDim.x) {
-    const int i = (int)(n % NX), j = (int)((n / NX) % NY), k = (int)(n / (NX * NY));
+    int i, j, k;
+    grid_ijk((unsigned)n, g.NX, g.NY, &i, &j, &k);
     const int s = slot_at(g, i, j, k);
     const size_t head[3] = {n + 1, n + NX, n + NX * NY};
     const bool has[3] = {i + 1 < g.NX, j + 1 < g.NY, k + 1 < g.NZ};
@@ -758,7 +763,7 @@ k_energy_grad_sigma(const unsigned char *__restrict__ mask, const double *__rest
     double acc = 0.0;
     if (mask[v]) {
       int i, j, k;
-      voxel_ijk(v, nx, ny, &i, &j, &k);
+      grid_ijk((unsigned)v, nx, ny, &i, &j, &k);
       const size_t n = (size_t)k * NXY + (size_t)j * NX + i;
 #pragma unroll
       for (int pq = 0; pq < 4; ++pq) {
@@ -1071,13 +1076,13 @@ void launch_rhs(const Grid &g, const double *gx, const double *a, double *b,
   if (g.nb) k_rhs<<<dim3(g.nb, nk), NT, 0, st>>>(g, gx, a, b, status);
 }
 template <typename T>
-void launch_scatter(const Grid &g, const T *x, const int *comp, double *psi,
+void launch_scatter(const Grid &g, const T *x, const unsigned *ubits, double *psi,
                     cudaStream_t st, int nk) {
   size_t NN = (size_t)g.NX * g.NY * g.NZ;
   size_t blocks = (NN + 255) / 256;
   if (blocks > 152 * 64) blocks = 152 * 64;
   if (blocks == 0) blocks = 1;
-  pdl(k_scatter<T>, dim3((int)blocks, nk), 256, st)(g, x, comp, psi);
+  pdl(k_scatter<T>, dim3((int)blocks, nk), 256, st)(g, x, ubits, psi);
 }
 void launch_gather(const Grid &g, const double *psi, const int *comp, double *x,
                    cudaStream_t st) {
@@ -1174,7 +1179,7 @@ void launch_energy_grads(const Grid &g, const double *gx, const unsigned char *m
   template void launch_dot<T>(int, const T *, const T *, const unsigned *,     \
                               Scalars *, double *, int, cudaStream_t, int,     \
                               size_t);                                         \
-  template void launch_scatter<T>(const Grid &, const T *, const int *,        \
+  template void launch_scatter<T>(const Grid &, const T *, const unsigned *,   \
                                   double *, cudaStream_t, int);
 INST_K(double)
 INST_K(float)
