@@ -727,7 +727,7 @@ spfd_status build_impl(spfd_ctx *c, const double *sigma) {
   // scratch) while the main stream inverts the coarsest level.  The side
   // streams fork from the main stream before the coarsest level, but their
   // kernels are enqueued after the inverse's cooperative launch: launched
-  // first, the inverse takes its SM slots (a quarter of each SM's threads),
+  // first, the inverse takes its SM slots (a 256-thread block on most SMs),
   // and the power iterations fill the rest beside it instead of holding
   // every SM until they end.
   {

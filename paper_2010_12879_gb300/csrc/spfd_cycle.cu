@@ -6,9 +6,10 @@
 // geometric operator-dependent V-cycle that replaces it.  All are
 // bandwidth-bound stencil or transfer sweeps (the FP64 forms approach the
 // FP64 pipe's rate); none is a dense contraction, so no tensor-core path is
-// used.  One block handles one 8x8x8 brick: two (FP64) or four (FP32) nodes
-// per thread without shared memory on level 0, one node per thread with a shared tile on the
-// 27-point levels (spfd_tile.cuh).
+// used.  One block handles one 8x8x8 brick: two or four nodes of an x-row per
+// thread without shared memory on level 0, one node per thread with a shared tile on
+// the large 27-point levels (spfd_tile.cuh); the small ones run as quarter
+// bricks (spfd_slab.cu).
 #include "spfd_internal.cuh"
 #include "spfd_reduce.cuh"
 #include "spfd_tile.cuh"
@@ -19,10 +20,7 @@ constexpr int CS_THREADS = 128;  // threads per block of the coarsest solve
 
 // ------------------------------------------------------------ smoothers
 // Level 0 (7-point): r = b - A x, and the weighted-Jacobi sweep
-// x_out = x + omega D^-1 (b - A x), on the row mapping.  (The level-0 row
-// list that k_apply_dot uses in FP64 made these two slower: they issue
-// fewer FP64 instructions per row, and the extra dependent load of the list
-// entry and the looser brick locality cost more than the skipped rows.)
+// x_out = x + omega D^-1 (b - A x), on the row mapping.
 template <typename T, typename C, int ORD>
 __global__ void __launch_bounds__(row_threads<T>(), row_min_blocks<T>())
 k_residual7(Grid g, const C *__restrict__ gx, const T *__restrict__ diag,

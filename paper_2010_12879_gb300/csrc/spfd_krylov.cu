@@ -2,7 +2,7 @@
 // side of Eq. 3, the Psi scatter and the |E| of Eq. 1.
 //
 // Reductions finish on the device: blocks write partial sums, and either the
-// last block to arrive (ticket counter) or a one-block finishing kernel adds
+// last block to arrive (ticket counter) or a one-cluster finishing kernel adds
 // them in a fixed order and updates the Krylov scalars in place, so the loop
 // needs no host round trip except the convergence test.
 //
