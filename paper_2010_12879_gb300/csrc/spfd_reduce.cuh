@@ -31,7 +31,10 @@ template <> struct Acc<float> {
 // and warp 0 adds them (lane l the values of threads l, l + 32, ..., then a
 // butterfly): NV * (warps + 4) FP64 warp instructions per block, against
 // 5 NV per warp plus 5 NV for a butterfly in every warp, on GB300's narrow
-// FP64 pipe.
+// FP64 pipe.  The NV chains of dependent additions run side by side and their
+// loads ahead of them (MT bounds the loop): the tail of a reduction is their
+// latency, once in each block and once more in the last one (32^3 sphere
+// solve 1107 -> 1082 us, 16 mm step 2058 -> 2037; no change at 2 mm).
 template <int NV, int MT = NT>
 __device__ __forceinline__ void block_sum(double (&v)[NV]) {
   __shared__ double sm[NV][MT];
@@ -42,13 +45,16 @@ __device__ __forceinline__ void block_sum(double (&v)[NV]) {
   __syncthreads();
   if (w == 0) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double a = sm[k][lane];
-      for (int i = 1; i < nw; ++i) a += sm[k][lane + 32 * i];
+    for (int k = 0; k < NV; ++k) v[k] = sm[k][lane];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-      v[k] = a;
-    }
+    for (int i = 1; i < MT / 32; ++i)
+      if (i < nw)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) v[k] += sm[k][lane + 32 * i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < NV; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
   }
   __syncthreads();
 }
