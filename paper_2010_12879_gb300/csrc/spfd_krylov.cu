@@ -94,6 +94,10 @@ k_finish_pairs(const double *__restrict__ pairs, int n, Scalars *sc, int first,
   const float2 *pp = reinterpret_cast<const float2 *>(pairs + (size_t)blockIdx.y * pstride);
   sc += blockIdx.y;
   if (NV == 1 && sc->frozen) return;  // the whole cluster: its operator wrote nothing
+  // the first block's shared memory may be written once that block has
+  // started: every block arrives here and waits before its store, so that the
+  // loads in between hide the barrier
+  cl.barrier_arrive();
   float hi[NV], lo[NV];
 #pragma unroll
   for (int k = 0; k < NV; ++k) hi[k] = lo[k] = 0.f;
@@ -116,6 +120,7 @@ k_finish_pairs(const double *__restrict__ pairs, int n, Scalars *sc, int first,
     }
   }
   __syncthreads();
+  cl.barrier_wait();
   if (w == 0) {
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
