@@ -232,10 +232,16 @@ k_pct_collect(const unsigned char *__restrict__ mask, const double *__restrict__
 }
 
 // 4a. Digit histogram of the listed keys that match their group's prefix.
+// *listed entries were written; want, as many as the buckets counted, when
+// the inputs did not change during the call.  Fewer are flagged, and no entry
+// past them is read: its group would be any number.
 __global__ void __launch_bounds__(PT)
 k_pct_hist(const unsigned long long *__restrict__ key, const int *__restrict__ kgrp,
-           unsigned long long n, const PctGroup *__restrict__ grp, int shift, int width,
-           unsigned *__restrict__ hist) {
+           const unsigned long long *__restrict__ listed, unsigned long long want,
+           const PctGroup *__restrict__ grp, int shift, int width,
+           unsigned *__restrict__ hist, int *status) {
+  const unsigned long long n = min(*listed, want);
+  if (n != want && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, PCT_BAD_RANK);
   const int hi = shift + width;
   const unsigned dmask = (1u << width) - 1u;
   const unsigned long long stride = (unsigned long long)gridDim.x * PT;
@@ -358,8 +364,8 @@ extern "C" spfd_status spfd_percentile(spfd_ctx *ctx, const double *E_dev,
     for (int left = 63 - width; left > 0;) {
       const int w = std::min(left, 13), shift = left - w;
       SPFD_LAUNCH(c, "percentile_hist", false, 2, 12.0 * listed, 0,
-                  (k_pct_hist<<<hgrid, PT, 0, st>>>(c->pct_keys, c->pct_keyg, listed, grp, shift,
-                                                    w, c->pct_hist),
+                  (k_pct_hist<<<hgrid, PT, 0, st>>>(c->pct_keys, c->pct_keyg, cursor, listed,
+                                                    grp, shift, w, c->pct_hist, status),
                    k_pct_select<<<G, PT, 0, st>>>(c->pct_hist, grp, shift, w, status)));
       left = shift;
     }
@@ -369,8 +375,8 @@ extern "C" spfd_status spfd_percentile(spfd_ctx *ctx, const double *E_dev,
   }
   TRY(prof_flush(c));
   if (*hstatus & PCT_BAD_RANK) {
-    // a row of the later digits may be left behind: allocate (and clear) anew
-    c->pct_gcap = 0;
+    // a row of the later digits may be left behind
+    CU(cudaMemsetAsync(c->pct_hist, 0, (size_t)c->pct_gcap * PCT_BINS * sizeof(unsigned), st));
     return fail(SPFD_EINTERNAL, "percentile selection lost its rank (|E| or labels "
                                 "changed during the call?)");
   }
