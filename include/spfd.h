@@ -288,9 +288,11 @@ spfd_status spfd_tree_cotree(const double *b_dev, int nx, int ny, int nz, int j0
  *   values_host  host output of n_labels + 1 entries: tissues 0..n_labels-1,
  *                then the whole body (NaN for a group without voxels).
  *   counts_host  optional host output of n_labels + 1 voxel counts.
- * Allocates scratch on first use (16 MB, 32 KB per group and 12 bytes for
- * each value that shares its group's first digit, a few per cent of the
- * conducting voxels) and keeps it; synchronises the stream. */
+ * |E| and the labels are read in several passes and must not change during
+ * the call (SPFD_EINTERNAL where that is noticed).
+ * Allocates scratch on first use (up to 20 MB of counters, 32 KB per group
+ * and a list of keys, 15 bytes for each, at most an eighth of the conducting
+ * voxels or 65536) and keeps it; synchronises the stream. */
 spfd_status spfd_percentile(spfd_ctx *ctx, const double *E_dev, const int32_t *labels_dev,
                             int n_labels, double p, double *values_host,
                             int64_t *counts_host);

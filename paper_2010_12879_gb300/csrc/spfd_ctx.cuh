@@ -171,12 +171,13 @@ struct spfd_ctx {
   const double *gJ_cur = nullptr;
   double *ev_stage = nullptr, *gj_stage = nullptr, *lam_stage = nullptr;
   // scratch of spfd_percentile (allocated on first use, grown on demand): the
-  // first digit's table, the later digits', the groups with their pinned
+  // field digits' table, the later digits', the groups with their pinned
   // mirror, and the listed keys with their groups
   unsigned *pct_first = nullptr, *pct_hist = nullptr;
   unsigned long long *pct_grp = nullptr, *pct_hgrp = nullptr, *pct_keys = nullptr;
   int *pct_keyg = nullptr;
   int pct_gcap = 0;
+  size_t pct_tcap = 0;  // counters of pct_first
   long long pct_keycap = 0, pct_nc = 0;  // pct_nc: conducting voxels seen last call
   // block orders chosen by the autotuner for batched launches: per batch
   // size, TF_COUNT x (levels) entries of 0 or 1; ord points at the table of
