@@ -13,7 +13,8 @@
 //               CG (operator with FP32 conductances, V-cycle with BF16
 //               finest-level conductances and FP32 accumulation) solves
 //               A d = r to a modest relative accuracy, x += d in FP64.
-//               Dot products accumulate in FP64; the coarsest solve is FP64.
+//               Dot products accumulate in FP64, or in FP32 parts that carry
+//               their rounding errors; the coarsest solve is FP64.
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>

@@ -9,8 +9,8 @@
 // GB300's FP64 pipe retires about one FP64 operation per 11 bytes of HBM
 // traffic, so FP32 kernels here keep every per-element operation in FP32:
 // scalars arrive pre-converted (alpha_f, beta_f, ...) and dot products sum
-// per thread in compensated (Kahan) FP32 before the FP64 tree across threads
-// and blocks.
+// per thread in compensated FP32, whose errors are carried along (pairs, Sum3)
+// up to the block's total, the first FP64 value.
 #include <algorithm>
 
 #include <cooperative_groups.h>
@@ -76,10 +76,14 @@ k_apply_dot(Grid g, const T *__restrict__ gx, const T *__restrict__ diag,
 
 // The n (times NV) pairs of an FP32 row kernel added, and the scalars set: NV =
 // 1 p.q and alpha, NV = 2 r.z, beta and the mean of z.  One cluster of eight
-// blocks per right-hand side: the threads add pairs without rounding error,
-// each block's total is widened to FP64 and passed to the first block through
-// its shared memory.  A grid with a ticket (fence, atomic, second round
-// through L2) took 7.4 us for 89,000 pairs and 12.3 us for twice as many.
+// blocks per right-hand side: the threads add pairs in three FP32 parts
+// (Sum3, at least as accurate as FP64 additions, of which 178,000 pairs would
+// take 11 us on eight SMs' FP64 pipes), each block's total is widened to FP64
+// and passed to the first block through its shared memory.  A grid with a
+// ticket (fence, atomic, second round through L2) and FP64 additions took 7.4
+// us for 89,000 pairs and 12.3 us for twice as many.  Two FP32 parts would take
+// 0.3 % less of a 2 mm mixed step (16.96 against 17.01 ms), with 48 bits.
+// A total beyond FP32's range, or not a number, is added again in FP64.
 constexpr int FP_CLUSTER = 8, FP_THREADS = 1024;
 template <int NV>
 __global__ void __cluster_dims__(FP_CLUSTER, 1, 1) __launch_bounds__(FP_THREADS)
@@ -89,7 +93,7 @@ k_finish_pairs(const double *__restrict__ pairs, int n, Scalars *sc, int first,
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   __shared__ double all[FP_CLUSTER][NV];
-  __shared__ float sh[32][NV], sl[32][NV];
+  __shared__ Sum3 part[32][NV];
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const float2 *pp = reinterpret_cast<const float2 *>(pairs + (size_t)blockIdx.y * pstride);
   sc += blockIdx.y;
@@ -98,49 +102,53 @@ k_finish_pairs(const double *__restrict__ pairs, int n, Scalars *sc, int first,
   // started: every block arrives here and waits before its store, so that the
   // loads in between hide the barrier
   cl.barrier_arrive();
-  float hi[NV], lo[NV];
+  Sum3 a[NV];
 #pragma unroll
-  for (int k = 0; k < NV; ++k) hi[k] = lo[k] = 0.f;
+  for (int k = 0; k < NV; ++k) a[k] = Sum3{0.f, 0.f, 0.f};
 #pragma unroll 4
   for (int i = blockIdx.x * FP_THREADS + t; i < n; i += FP_CLUSTER * FP_THREADS)
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
       const float2 q = pp[(size_t)NV * i + k];
-      two_sum_add(hi[k], lo[k], q.x, q.y);
+      sum3_add(a[k], q.x, q.y, 0.f);
     }
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-      two_sum_add(hi[k], lo[k], __shfl_xor_sync(0xffffffffu, hi[k], o),
-                  __shfl_xor_sync(0xffffffffu, lo[k], o));
-    if (lane == 0) {
-      sh[w][k] = hi[k];
-      sl[w][k] = lo[k];
-    }
+    sum3_warp(a[k]);
+    if (lane == 0) part[w][k] = a[k];
   }
   __syncthreads();
   cl.barrier_wait();
   if (w == 0) {
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
-      float h = sh[lane][k], l = sl[lane][k];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1)
-        two_sum_add(h, l, __shfl_xor_sync(0xffffffffu, h, o), __shfl_xor_sync(0xffffffffu, l, o));
+      a[k] = part[lane][k];
+      sum3_warp(a[k]);
       if (lane == 0)
-        cl.map_shared_rank(&all[0][0], 0)[NV * cl.block_rank() + k] = (double)h + (double)l;
+        cl.map_shared_rank(&all[0][0], 0)[NV * cl.block_rank() + k] = sum3_value(a[k]);
     }
   }
   cl.sync();
-  if (cl.block_rank() == 0 && t == 0) {
+  if (cl.block_rank() == 0 && w == 0) {
     double tot[2] = {0.0, 0.0};
 #pragma unroll
-    for (int k = 0; k < NV; ++k)
+    for (int k = 0; k < NV; ++k) {
 #pragma unroll
       for (int b = 0; b < FP_CLUSTER; ++b) tot[k] += all[b][k];
-    if constexpr (NV == 1) set_pq(sc, tot[0]);
-    else set_rz(sc, tot, first);
+      if (f64_nonfinite(tot[k])) {
+        tot[k] = 0.0;
+        for (int i = lane; i < n; i += 32) {
+          const float2 q = pp[(size_t)NV * i + k];
+          tot[k] += (double)q.x + (double)q.y;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) tot[k] += __shfl_xor_sync(0xffffffffu, tot[k], o);
+      }
+    }
+    if (lane == 0) {
+      if constexpr (NV == 1) set_pq(sc, tot[0]);
+      else set_rz(sc, tot, first);
+    }
   }
 }
 

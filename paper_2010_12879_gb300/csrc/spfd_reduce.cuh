@@ -108,6 +108,36 @@ __device__ __forceinline__ void two_sum_add(float &hi, float &lo, float oh, floa
   lo = lo + ol + e;
 }
 
+// A sum of three FP32 parts h + m + l, for adding many FP32 pairs without
+// the FP64 pipe and with no larger error than FP64 additions: the rounding
+// errors of the high parts go to the middle ones, and theirs to the low ones,
+// whose own are below (c 2^-24)^3 of the sum of magnitudes after c additions
+// in a row.
+struct Sum3 {
+  float h, m, l;
+};
+__host__ __device__ __forceinline__ float two_sum(float a, float b, float &err) {
+  const float s = a + b, bb = s - a;
+  err = (a - (s - bb)) + (b - bb);
+  return s;
+}
+__host__ __device__ __forceinline__ void sum3_add(Sum3 &t, float h, float m, float l) {
+  float e1, e2, e3;
+  t.h = two_sum(t.h, h, e1);
+  t.m = two_sum(t.m, m, e2);
+  t.m = two_sum(t.m, e1, e3);
+  t.l = (t.l + l) + (e2 + e3);
+}
+__host__ __device__ __forceinline__ double sum3_value(const Sum3 &t) {
+  return (double)t.h + ((double)t.m + (double)t.l);
+}
+__device__ __forceinline__ void sum3_warp(Sum3 &t) {  // the warp's total in every lane
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    sum3_add(t, __shfl_xor_sync(0xffffffffu, t.h, o), __shfl_xor_sync(0xffffffffu, t.m, o),
+             __shfl_xor_sync(0xffffffffu, t.l, o));
+}
+
 // grid_sum for per-thread FP32 pairs (value hi + lo): the warps and the block
 // add them as TwoSum pairs in FP32, and only the block's total is widened to
 // FP64 (in thread 0).  An FP64 conversion or addition takes a 16-clock slot
