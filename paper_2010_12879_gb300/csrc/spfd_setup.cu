@@ -554,7 +554,7 @@ void launch_coarse_dense(const Grid &g, const double *op, bool k27, size_t S, co
 // After every pivot set has been swept once, B = A^-1.  D is inverted by
 // scalar Gauss-Jordan in shared memory: its pivots are Schur complements of
 // the SPD matrix, hence positive; a non-positive one raises DEV_BAD_PIVOT.
-// Sweeps run in one cooperative launch (k_gj_strips) or, for large m, one
+// Sweeps run in one cooperative launch (k_gj_strips) or, beyond GS_MAX, one
 // launch each (k_gj_block, where every block inverts D itself); the order of
 // every sum is the same in both.
 constexpr int GJ_B = 16;   // pivots per sweep
@@ -659,7 +659,7 @@ k_gj_block(const double *__restrict__ A, double *__restrict__ B, int m, int k0, 
 }
 
 // Every sweep in one cooperative launch, with a grid barrier between sweeps.
-// Block s updates the four columns 4s .. 4s + 3 over all rows, and one block
+// Block s updates the GW columns GW s .. over all rows, and one block
 // more forms the next sweep's D (its 16 x 16 entries updated as any other)
 // and inverts it meanwhile, so that the inversion's 16 dependent steps are
 // off the update's path and done once.  With a 32 x 32 tile per block, each
@@ -670,36 +670,43 @@ k_gj_block(const double *__restrict__ A, double *__restrict__ B, int m, int k0, 
 // dinv: two 16 x 16 buffers; bar: barrier counter and generation, zero at
 // launch.  Reads of the matrix go through L2 (ld.global.cg): other blocks
 // wrote it in the previous sweep.
-constexpr int GS_W = 4;                  // columns per block
-constexpr int GS_R = GJ_NT / GS_W;       // rows per pass of the block
+// GW = 4 spreads the pipe's work over all SMs up to about 600 unknowns.  From
+// 513 on M[., K] leaves room for one block an SM, so that m / 4 + 1 blocks
+// are not resident at once beyond 604 (152 SMs); GW = 8 halves their number
+// and serves up to GS_MAX: 605 unknowns 1.43 -> 1.13 ms against a launch per
+// sweep, 800 2.87 -> 1.84, 1000 4.90 -> 2.68 (600 with GW = 4: 0.76).
 constexpr int GS_K = 8;                  // rows per thread and chunk
 constexpr int GS_MAX = 1024;             // largest m (shared memory: 136 bytes per row)
+template <int GW> constexpr int gs_rows() { return GJ_NT / GW; }  // per pass of the block
 // rows up to the last chunk's end: a thread reads (and discards) U past row m
+template <int GW>
 constexpr size_t gs_smem(int m) {
-  return (size_t)((m + GS_R * GS_K - 1) / (GS_R * GS_K)) * (GS_R * GS_K) * (GJ_B + 1) *
-         sizeof(double);
+  constexpr int chunk = gs_rows<GW>() * GS_K;
+  return (size_t)((m + chunk - 1) / chunk) * chunk * (GJ_B + 1) * sizeof(double);
 }
 
-// Rows row0 + GS_R k (k < NK) of column j: v -= U W, in order l = 0..15.
-template <int NK>
+// Rows row0 + GR k (k < NK) of column j: v -= U W, in order l = 0..15.
+template <int NK, int GR>
 __device__ __forceinline__ void gs_update(const double *__restrict__ U, const double *wc,
                                           int wstride, int row0, double (&v)[GS_K]) {
 #pragma unroll
   for (int l = 0; l < GJ_B; ++l) {
     const double mc = wc[l * wstride];
 #pragma unroll
-    for (int k = 0; k < NK; ++k) v[k] -= U[(row0 + GS_R * k) * (GJ_B + 1) + l] * mc;
+    for (int k = 0; k < NK; ++k) v[k] -= U[(row0 + GR * k) * (GJ_B + 1) + l] * mc;
   }
 }
 
+template <int GW>
 __global__ void __launch_bounds__(GJ_NT)
 k_gj_strips(double *buf0, double *buf1, int m, double *dinv, int *status, unsigned *bar) {
+  constexpr int GR = gs_rows<GW>();
   extern __shared__ double U[];  // [m rounded up][GJ_B + 1]
   __shared__ GjPivots pv;
-  __shared__ double Ds[GJ_B][GJ_B + 1], W[GJ_B][GS_W], C[GJ_B][GS_W], Cn[GJ_B][GJ_B + 1];
+  __shared__ double Ds[GJ_B][GJ_B + 1], W[GJ_B][GW], C[GJ_B][GW], Cn[GJ_B][GJ_B + 1];
   const int t = threadIdx.x, a = t / GJ_B, b = t % GJ_B;
   const bool pivot = blockIdx.x == gridDim.x - 1;
-  const int j0 = blockIdx.x * GS_W, jj = t % GS_W, j = j0 + jj, rg = t / GS_W;
+  const int j0 = blockIdx.x * GW, jj = t % GW, j = j0 + jj, rg = t / GW;
   double *A = buf0, *B = buf1;
   if (pivot) {  // the first sweep's D^-1
     const int r = min(GJ_B, m);
@@ -734,8 +741,8 @@ k_gj_strips(double *buf0, double *buf1, int m, double *dinv, int *status, unsign
         dinv[((sw + 1) & 1) * GJ_NT + t] = pv.D[GJ_B & 1][a][b];
       }
     } else {
-      if (t < GJ_B * GS_W) {
-        const int l2 = t / GS_W;
+      if (t < GJ_B * GW) {
+        const int l2 = t / GW;
         C[l2][jj] = (l2 < r && j < m) ? __ldcg(&A[(size_t)(k0 + l2) * m + j]) : 0.0;
       }
 #pragma unroll 8
@@ -748,14 +755,14 @@ k_gj_strips(double *buf0, double *buf1, int m, double *dinv, int *status, unsign
       auto load = [&](int base) {
 #pragma unroll
         for (int k = 0; k < GS_K; ++k) {
-          const int i = base + rg + GS_R * k;
+          const int i = base + rg + GR * k;
           v[k] = (!kj && i < m && j < m) ? __ldcg(&A[(size_t)i * m + j]) : 0.0;
         }
       };
       load(0);
       __syncthreads();
-      if (t < GJ_B * GS_W) {
-        const int l = t / GS_W;
+      if (t < GJ_B * GW) {
+        const int l = t / GW;
         double w = 0.0;
 #pragma unroll
         for (int l2 = 0; l2 < GJ_B; ++l2) w += Ds[l][l2] * C[l2][jj];
@@ -763,19 +770,19 @@ k_gj_strips(double *buf0, double *buf1, int m, double *dinv, int *status, unsign
       }
       __syncthreads();
       const double *wc = kj ? &Ds[0][j - k0] : &W[0][jj];
-      const int ws = kj ? GJ_B + 1 : GS_W;
-      for (int base = 0; base < m; base += GS_R * GS_K) {
+      const int ws = kj ? GJ_B + 1 : GW;
+      for (int base = 0; base < m; base += GR * GS_K) {
         if (base) load(base);
-        // rows this warp has left, uniform: its first row and every GS_R-th
-        const int left = m - base - (t & ~31) / GS_W;
-        const int nk = left <= 0 ? 0 : (left + GS_R - 1) / GS_R;
-        if (nk >= GS_K) gs_update<GS_K>(U, wc, ws, base + rg, v);
-        else if (nk == GS_K - 1) gs_update<GS_K - 1>(U, wc, ws, base + rg, v);
-        else if (nk > GS_K / 2) gs_update<GS_K - 2>(U, wc, ws, base + rg, v);
-        else if (nk > 0) gs_update<GS_K / 2>(U, wc, ws, base + rg, v);
+        // rows this warp has left, uniform: its first row and every GR-th
+        const int left = m - base - (t & ~31) / GW;
+        const int nk = left <= 0 ? 0 : (left + GR - 1) / GR;
+        if (nk >= GS_K) gs_update<GS_K, GR>(U, wc, ws, base + rg, v);
+        else if (nk == GS_K - 1) gs_update<GS_K - 1, GR>(U, wc, ws, base + rg, v);
+        else if (nk > GS_K / 2) gs_update<GS_K - 2, GR>(U, wc, ws, base + rg, v);
+        else if (nk > 0) gs_update<GS_K / 2, GR>(U, wc, ws, base + rg, v);
 #pragma unroll
         for (int k = 0; k < GS_K; ++k) {
-          const int i = base + rg + GS_R * k;
+          const int i = base + rg + GR * k;
           if (i >= m || j >= m) continue;
           const bool ki = i >= k0 && i < k0 + r;
           B[(size_t)i * m + j] = ki ? wc[(i - k0) * ws] : v[k];
@@ -787,24 +794,29 @@ k_gj_strips(double *buf0, double *buf1, int m, double *dinv, int *status, unsign
   }
 }
 
-// Whether the m x m inverse runs as one cooperative launch: its blocks have
-// to be resident all at once.
-static bool gj_one_launch(int m) {
-  int dev = 0, nsm = 0, per_sm = 0, coop = 0;
+// The strips' width for which the m x m inverse runs as one cooperative launch
+// (its blocks have to be resident all at once), 0 when neither fits.
+template <int GW>
+static bool gj_fits(int m, int nsm) {
+  int per_sm = 0;
+  return cudaFuncSetAttribute(k_gj_strips<GW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)gs_smem<GW>(GS_MAX)) == cudaSuccess &&
+         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gj_strips<GW>, GJ_NT,
+                                                       gs_smem<GW>(m)) == cudaSuccess &&
+         (m + GW - 1) / GW + 1 <= per_sm * nsm;
+}
+static int gj_strip_width(int m) {
+  int dev = 0, nsm = 0, coop = 0, width = 0;
   if (m <= GS_MAX && cudaGetDevice(&dev) == cudaSuccess &&
       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
-      cudaFuncSetAttribute(k_gj_strips, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)gs_smem(GS_MAX)) == cudaSuccess &&
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gj_strips, GJ_NT, gs_smem(m)) ==
-          cudaSuccess)
-    return (m + GS_W - 1) / GS_W + 1 <= per_sm * nsm;
-  cudaGetLastError();
-  return false;
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop)
+    width = gj_fits<4>(m, nsm) ? 4 : gj_fits<8>(m, nsm) ? 8 : 0;
+  if (!width) cudaGetLastError();
+  return width;
 }
 
 // Kernel launches of launch_dense_inverse for an m x m matrix.
-int dense_inverse_launches(int m) { return gj_one_launch(m) ? 1 : (m + GJ_B - 1) / GJ_B; }
+int dense_inverse_launches(int m) { return gj_strip_width(m) ? 1 : (m + GJ_B - 1) / GJ_B; }
 
 // Inverts the SPD matrix in buf0 (m x m); returns the buffer holding A^-1
 // (buf0 or buf1, which serve as ping-pong buffers).  dinv: 512 doubles and
@@ -812,10 +824,11 @@ int dense_inverse_launches(int m) { return gj_one_launch(m) ? 1 : (m + GJ_B - 1)
 double *launch_dense_inverse(double *buf0, double *buf1, int m, double *dinv, int *status,
                              unsigned *bar, cudaStream_t st) {
   double *a = buf0, *b = buf1;
-  if (gj_one_launch(m)) {
+  if (const int width = gj_strip_width(m)) {
     void *args[] = {&buf0, &buf1, &m, &dinv, &status, &bar};
-    if (cudaLaunchCooperativeKernel((const void *)k_gj_strips, dim3((m + GS_W - 1) / GS_W + 1),
-                                    dim3(GJ_NT), args, gs_smem(m), st) == cudaSuccess)
+    const void *kernel = width == 4 ? (const void *)k_gj_strips<4> : (const void *)k_gj_strips<8>;
+    if (cudaLaunchCooperativeKernel(kernel, dim3((m + width - 1) / width + 1), dim3(GJ_NT), args,
+                                    width == 4 ? gs_smem<4>(m) : gs_smem<8>(m), st) == cudaSuccess)
       return ((m + GJ_B - 1) / GJ_B) % 2 ? buf1 : buf0;
     cudaGetLastError();  // not launched: sweep launch by launch instead
   }
