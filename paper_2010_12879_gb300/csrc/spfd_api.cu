@@ -1008,10 +1008,15 @@ static spfd_status solve_mixed(spfd_ctx *c, double tol, spfd_info *out, int nk =
 // level's x, b, r, t, the FP64 Krylov vectors, the scalars (each with
 // inv_ndof), the reduction scratch and the component sums.  New vectors are
 // zeroed (slots that are not unknowns must read 0).  Synchronises the stream.
-static spfd_status ensure_batch(spfd_ctx *c, int k) {
+// The old buffers go before the new ones come, so a failed growth leaves some
+// of them missing: the capacity is 0 then, and whatever uses them next grows
+// them first.
+spfd_status ensure_batch(spfd_ctx *c, int k) {
   if (k <= c->kcap) return SPFD_OK;
   cudaStream_t st = c->stream;
   TRY(sync_check(c, "batch buffers"));
+  c->kcap = 0;
+  ++c->gen;  // solve buffers move: captured graphs must be captured again
   auto grow = [&](double *&v, size_t n) -> spfd_status {
     dfree(c, v);
     TRY(dalloc(c, &v, n));
@@ -1041,8 +1046,11 @@ static spfd_status ensure_batch(spfd_ctx *c, int k) {
   TRY(grow(c->partials, c->pstride * k));
   if (c->ncomp > 1) TRY(grow(c->csum, (size_t)c->cstride * k));
   Scalars *sc = nullptr, *hsc = nullptr;
+  HostFlag *hflag = nullptr;
   TRY(dalloc(c, &sc, k));
   TRY(halloc(c, &hsc, k));
+  TRY(halloc(c, &hflag, k));
+  memset(hflag, 0, (size_t)k * sizeof(HostFlag));
   memset(hsc, 0, (size_t)k * sizeof(Scalars));
   const double inv_ndof = c->ndof ? 1.0 / (double)c->ndof : 0.0;
   for (int j = 0; j < k; ++j) hsc[j].inv_ndof = inv_ndof;
@@ -1050,10 +1058,8 @@ static spfd_status ensure_batch(spfd_ctx *c, int k) {
   TRY(sync_check(c, "batch scalars"));
   dfree(c, c->sc);
   c->sc = sc;
-  ++c->gen;  // solve buffers moved: captured graphs must be captured again
   c->hsc = hsc;
-  TRY(halloc(c, &c->hflag, k));
-  memset(c->hflag, 0, (size_t)k * sizeof(HostFlag));
+  c->hflag = hflag;
   c->kcap = k;
   return SPFD_OK;
 }
@@ -1069,7 +1075,7 @@ static spfd_status solve_device(spfd_ctx *c, const double *a_dev, double tol,
   const size_t NNs = (size_t)(c->nx + 1) * (c->ny + 1) * (c->nz + 1);
   std::vector<spfd_info> res(nk, c->info);
   const int64_t launches0 = c->launch_count;
-  if (nk > 1 && c->ndof > 0) TRY(ensure_batch(c, nk));
+  if (c->ndof > 0) TRY(ensure_batch(c, nk));
   const signed char *orders = nullptr;
   TRY(batch_orders(c, nk, &orders));
   CU(cudaEventRecord(c->ev0, st));
@@ -1136,6 +1142,7 @@ extern "C" spfd_status spfd_energy_grad(spfd_ctx *ctx, const double *a_dev,
   Level &l0 = c->L[0];
   const size_t nv = (size_t)c->nx * c->ny * c->nz;
   const size_t NN = (size_t)(c->nx + 1) * (c->ny + 1) * (c->nz + 1);
+  if (c->ndof > 0) TRY(ensure_batch(c, 1));
   if (!c->ev_stage) TRY(dalloc(c, &c->ev_stage, 3 * nv));
   if (!c->gj_stage) TRY(dalloc(c, &c->gj_stage, 3 * NN));
   if (!c->lam_stage) TRY(dalloc(c, &c->lam_stage, NN));

@@ -155,7 +155,7 @@ struct spfd_ctx {
   size_t pstride = 0;
   // right-hand sides the per-RHS buffers hold (level vectors, Krylov
   // vectors, scalars, partials, component sums); grown by batched solves
-  int kcap = 1;
+  int kcap = 1;  // 0 after a growth that failed (ensure_batch)
   // generation of the solve buffers: bumped whenever they are reallocated,
   // so that graphs captured over them know to capture again
   uint64_t gen = 0;
@@ -299,6 +299,11 @@ spfd_status prof_flush(spfd_ctx *c);
 inline int block_order(const spfd_ctx *c, int fam, int l) {
   return c->ord ? c->ord[fam * (int)c->L.size() + l] : 0;
 }
+
+// Per-right-hand-side buffers for at least k of them (spfd_api.cu); at once
+// when they are there.  Called before anything uses them, since a growth that
+// failed left none.
+spfd_status ensure_batch(spfd_ctx *c, int k);
 
 // Solve steps shared by the host-driven solves (spfd_api.cu) and the
 // captured, device-driven ones (spfd_graph.cu).  All of them only enqueue

@@ -570,6 +570,8 @@ void release_graph(spfd_group *g) {
 spfd_status capture_group(spfd_group *g, const double *const *a, double *const *psi) {
   release_graph(g);
   const int n = (int)g->ctx.size();
+  for (spfd_ctx *c : g->ctx)
+    if (c->ndof > 0) TRY(ensure_batch(c, 1));
   g->rhs_node.assign(n, nullptr);
   g->scatter_node.assign(n, nullptr);
   std::vector<cudaStream_t> saved(n);
