@@ -79,10 +79,10 @@ k_apply_dot(Grid g, const T *__restrict__ gx, const T *__restrict__ diag,
 // blocks per right-hand side: the threads add pairs in three FP32 parts
 // (Sum3, at least as accurate as FP64 additions, of which 178,000 pairs would
 // take 11 us on eight SMs' FP64 pipes), each block's total is widened to FP64
-// and passed to the first block through its shared memory.  A grid with a
-// ticket (fence, atomic, second round through L2) and FP64 additions took 7.4
-// us for 89,000 pairs and 12.3 us for twice as many.  Two FP32 parts would take
-// 0.3 % less of a 2 mm mixed step (16.96 against 17.01 ms), with 48 bits.
+// and passed to the first block through its shared memory.  Timeline of a 2 mm
+// mixed solve, us for 89,000 pairs and for twice as many: a grid with a ticket
+// (fence, atomic, second round through L2) and FP64 additions 10.7 and 17.2,
+// two FP32 parts (48 bits) 8.4 and 9.3, this 9.0 and 11.6.
 // A total beyond FP32's range, or not a number, is added again in FP64.
 constexpr int FP_CLUSTER = 8, FP_THREADS = 1024;
 template <int NV>
